@@ -37,6 +37,7 @@ struct lbmp_ctx {
   int nsm = 1;                           // SMs of the device
   bool staged = true;            // staged kernel (else direct or wide)
   bool wide = false;             // wide FP16 kernel
+  bool fused = false;            // lbmp_step pairs its steps (two per launch)
   bool sr = false;
   bool fields_set = false;
   int64_t steps = 0;
@@ -48,8 +49,10 @@ struct lbmp_ctx {
   int alloc_count = 0;
   int fault_alloc_at = 0;       // simulated allocation failure (testing)
   int drop_tile = -1;           // withheld tile of the staged kernel (testing)
-  // step graphs: [l][cur] replays 2^l steps starting from buffer cur
+  // step graphs: [l][cur] replays 2^l launches starting from buffer cur (of
+  // two steps each with `fused`); odd[cur] the single step left over then
   cudaGraphExec_t graph[6][2] = {};
+  cudaGraphExec_t odd[2] = {};
 
   lbmp::StepArgs args() const {
     lbmp::StepArgs a;

@@ -1,0 +1,100 @@
+// Launches of the two-step kernel (fused.cuh).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "fused.cuh"
+#include "kernels.h"
+
+namespace lbmp {
+
+// Strips and segments of a launch: one warp per strip and segment.  A warp's
+// time is that of its seg + 2 rows (the two halo rows run the first level
+// only), so small segments cost redundant rows and large ones leave the last
+// wave uneven.  w waves of resident warps cost about 0.7 + w / 2 up to one (a
+// partly filled chip runs each row faster), 2.2 up to two, w + 0.25 beyond:
+// fitted to sweeps of seg at 512^2 .. 4096^2, where the choice is within 3% of
+// the best seg measured (1024^2: 6 rows 10.2 us a step, 5 rows 11.8; 4096^2
+// FP32: 28 rows 108.5, one wave of 82 rows 121).
+struct FusedPlan {
+  int strips, seg, tasks;
+};
+template <class C>
+static FusedPlan fused_plan(int nx, int rows, int nsm) {
+  const double cap = (double)nsm * C::kBlocks * kFusedWarps;
+  const int strips = fused_interior_strips<C>(nx) + 1;
+  const int most = (int)std::max(1.0, std::min((double)rows, 8.0 * cap / strips));
+  FusedPlan best{strips, rows, strips};
+  double best_cost = -1.0;
+  for (int parts = 1; parts <= most; ++parts) {
+    const int seg = (rows + parts - 1) / parts;
+    const int tasks = strips * ((rows + seg - 1) / seg);
+    const double w = tasks / cap;
+    const double cost = (seg + 2) * (w <= 1.0 ? 0.7 + 0.5 * w : (w <= 2.0 ? 2.2 : w + 0.25));
+    if (best_cost < 0.0 || cost < best_cost) {
+      best_cost = cost;
+      best = {strips, seg, tasks};
+    }
+  }
+  return best;
+}
+
+// Where two steps per launch are the faster form.  FP16 storage: everywhere
+// (against the staged kernel 64 x 33: 9.8 -> 2.4 us a step, 512^2 6.4 -> 4.9,
+// 4096^2 112.5 -> 105).  FP32: the direct kernel needs fewer rows in a row on
+// small lattices (512^2: 4.5 us against 4.7; 768^2: 7.6 against 7.2; 4096^2: 190
+// against 109), with a dynamic Kn up to about 10^6 nodes (768^2: 8.8 against 10.0;
+// 1024^2: 13.5 against 11.8).
+bool fused_covers(int storage, bool dyn, int nx, int ny) {
+  if (nx < FusedCfg<StoreF32, 1, false>::kCols || ny < kFusedMinNy) return false;
+  return storage != 0 || (long long)nx * ny >= (dyn ? 1000000 : 500000);
+}
+
+template <class S, bool SR, bool DYN, bool MOM, bool FORCH, int Q>
+static cudaError_t launch_fused_q(const StepArgs &a, int rows, const void *fin, void *fout,
+                                  const float2 *med, const unsigned long long *tctr, int k,
+                                  const FusedPlan &plan, float *mom1, float *mom2, cudaStream_t s) {
+  using C = FusedCfg<S, Q, DYN>;
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>,
+                           cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+  if (attr != cudaSuccess) return attr;
+  fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>
+      <<<(plan.tasks + kFusedWarps - 1) / kFusedWarps, kFusedWarps * 32, C::kSmemBytes, s>>>(
+          a, (const typename S::T *)fin, (typename S::T *)fout, med, tctr, k, rows, plan.seg,
+          plan.strips, plan.tasks, mom1, mom2);
+  return cudaGetLastError();
+}
+
+template <class S, bool SR, bool DYN, bool MOM>
+static cudaError_t launch_fused_t(const StepArgs &a, int rows, const void *fin, void *fout,
+                                  const float2 *med, const unsigned long long *tctr, int k,
+                                  int nsm, float *mom1, float *mom2, cudaStream_t s) {
+  using C1 = FusedCfg<S, 1, DYN>;
+  using C2 = FusedCfg<S, 2, DYN>;
+  // two pairs a lane spend fewer instructions a node, one pair a lane spreads
+  // a small lattice over more warps: 768^2 FP32 7.8 / 7.2 us a step, 1024^2
+  // 10.2 / 10.5, 1531 x 1153 14.1 / 17.0, 4096^2 108.5 / 119
+  const bool wide = a.nx >= C2::kCols && (long long)a.nx * rows >= 1000000;
+  const FusedPlan p = wide ? fused_plan<C2>(a.nx, rows, nsm) : fused_plan<C1>(a.nx, rows, nsm);
+#define LBMP_FUSED(FORCH, Q) \
+  launch_fused_q<S, SR, DYN, MOM, FORCH, Q>(a, rows, fin, fout, med, tctr, k, p, mom1, mom2, s)
+  if (a.forch) return wide ? LBMP_FUSED(true, 2) : LBMP_FUSED(true, 1);
+  return wide ? LBMP_FUSED(false, 2) : LBMP_FUSED(false, 1);
+#undef LBMP_FUSED
+}
+
+cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
+                         void *fout, const float2 *med, const unsigned long long *tctr, int k,
+                         int nsm, cudaStream_t s) {
+  const bool dyn = a.kn0 != nullptr;
+#define LBMP_FUSED(S, SR, DYN) \
+  launch_fused_t<S, SR, DYN, false>(a, rows, fin, fout, med, tctr, k, nsm, nullptr, nullptr, s)
+  if (storage == 0)
+    return dyn ? LBMP_FUSED(StoreF32, false, true) : LBMP_FUSED(StoreF32, false, false);
+  if (sr) return dyn ? LBMP_FUSED(StoreF16, true, true) : LBMP_FUSED(StoreF16, true, false);
+  return dyn ? LBMP_FUSED(StoreF16, false, true) : LBMP_FUSED(StoreF16, false, false);
+#undef LBMP_FUSED
+}
+
+}  // namespace lbmp

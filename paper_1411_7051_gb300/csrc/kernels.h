@@ -74,6 +74,14 @@ cudaError_t prepare_staged();
 cudaError_t launch_staged(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                           void *fout, const float2 *med, const unsigned long long *tctr, int k,
                           unsigned *err, int nsm, cudaStream_t s);
+// Two time steps in one launch (fused.cuh), bit for bit those of the
+// single-step kernels (FP16 with stochastic rounding: of the staged one),
+// with the rounding bits of time levels *tctr + k and *tctr + k + 1.
+// fused_covers(): the lattices on which lbmp_step pairs its steps.
+bool fused_covers(int storage, bool dyn, int nx, int ny);
+cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
+                         void *fout, const float2 *med, const unsigned long long *tctr, int k,
+                         int nsm, cudaStream_t s);
 // Store msg as the calling thread's lbmp_last_error() text.
 void set_last_error(const char *msg);
 

@@ -304,33 +304,34 @@ using NodeState = NodeStateT<float>;
 // Velocity and force of a permeable node (eps > 0): v = m / rho + eps G / 2,
 // u = v / (c0 + sqrt(c0^2 + c1 |v|)) (Eq. 17 when c1 = 0, i.e. without the
 // Forchheimer term), F = eps G - (eps nu / k_a + eps F_eps |u| / sqrt(k_a)) u
-// (Eq. 2).  c = 1 / (S rho).
-template <class V>
+// (Eq. 2).  c = 1 / (S rho).  The drag is formed with its sign reversed
+// (the packed operands have no negation): the same bits, no extra operation.
+template <bool SCALED = true, class V>
 __device__ __forceinline__ void porous_state(NodeStateT<V> &s, V eps, V inv_k, V c,
                                              const StepArgs &a) {
   s.ieps = vrcp(eps);
   const V eGx = vmul(eps, vsplat<V>(a.Gx)), eGy = vmul(eps, vsplat<V>(a.Gy));
   const V vx = vfma(vsplat<V>(0.5f), eGx, vmul(s.mx, c));
   const V vy = vfma(vsplat<V>(0.5f), eGy, vmul(s.my, c));
-  const V darcy = vmul(vmul(eps, vsplat<V>(a.nu)), inv_k);  // eps nu / k_a
-  const V c0 = vfma(vsplat<V>(0.25f), darcy, vsplat<V>(0.5f));  // (1 + eps nu / (2 k_a)) / 2
-  V idn, drag;
+  const V mdarcy = vmul(vmul(eps, vsplat<V>(-a.nu)), inv_k);  // -eps nu / k_a
+  const V c0 = vfma(vsplat<V>(-0.25f), mdarcy, vsplat<V>(0.5f));  // (1 + eps nu / (2 k_a)) / 2
+  V idn, mdrag;
   if (a.forch) {
     // c1 = eps F_eps / (2 sqrt(k_a)) with F_eps = 1.75 / sqrt(150 eps^3)
     const V c1 = vmul(vsplat<V>(a.fe_half), vsqrt(vmul(inv_k, s.ieps)));
     const V vmag = vsqrt(vfma(vx, vx, vmul(vy, vy)));
     idn = vrcp(vadd(c0, vsqrt(vfma(c0, c0, vmul(c1, vmag)))));
-    // eps nu / k_a + eps F_eps |u| / sqrt(k_a)
-    drag = vfma(vmul(vsplat<V>(2.0f), c1), vmul(vmag, idn), darcy);
+    // -(eps nu / k_a + eps F_eps |u| / sqrt(k_a))
+    mdrag = vfma(vmul(vsplat<V>(-2.0f), c1), vmul(vmag, idn), mdarcy);
   } else {
     idn = vrcp(vmul(vsplat<V>(2.0f), c0));
-    drag = darcy;
+    mdrag = mdarcy;
   }
   s.ux = vmul(vx, idn);
   s.uy = vmul(vy, idn);
-  s.Fx = vfma(vneg(drag), s.ux, eGx);
-  s.Fy = vfma(vneg(drag), s.uy, eGy);
-  const V rs = vmul(s.rho, vsplat<V>(a.scale));
+  s.Fx = vfma(mdrag, s.ux, eGx);
+  s.Fy = vfma(mdrag, s.uy, eGy);
+  const V rs = SCALED ? vmul(s.rho, vsplat<V>(a.scale)) : s.rho;
   s.rFx = vmul(rs, s.Fx);
   s.rFy = vmul(rs, s.Fy);
 }
@@ -387,21 +388,50 @@ __device__ __forceinline__ float2 kn_power(float2 K) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(t.y) : "f"(y_hi.y));
   return vfma(vmul(t, vsplat<float2>(0.69314718f)), y_lo, t);
 }
-__device__ __forceinline__ float2 dynamic_inv_k(float2 inv_k, float2 drho_s, float2 kn0,
-                                                const StepArgs &a) {
+// Kn of a pair at its current pressure.
+__device__ __forceinline__ float2 dynamic_kn(float2 drho_s, float2 kn0, const StepArgs &a) {
   const float2 q = vfma(vsplat<float2>(a.kn_beta), vmul(drho_s, vsplat<float2>(a.inv_scale)),
                         vsplat<float2>(1.0f));
-  const float2 kn = div_newton(kn0, q);
-  const bool common = a.kn_model == 0 && kn.x >= 1.17549435e-38f && kn.x <= 1e12f &&
-                      kn.y >= 1.17549435e-38f && kn.y <= 1e12f;
-  if (!common)  // the one-node form, lane by lane
-    return make_float2(inv_ka_dynamic(inv_k.x, kn.x, a.kn_model),
-                       inv_ka_dynamic(inv_k.y, kn.y, a.kn_model));
+  return div_newton(kn0, q);
+}
+// Whether both lanes take the fraction of Eq. 6-7 (the other cases of
+// inv_ka_dynamic are handled lane by lane).
+__device__ __forceinline__ bool kn_common(float2 kn, const StepArgs &a) {
+  return a.kn_model == 0 && kn.x >= 1.17549435e-38f && kn.x <= 1e12f &&
+         kn.y >= 1.17549435e-38f && kn.y <= 1e12f;
+}
+__device__ __forceinline__ float2 inv_ka_common(float2 inv_k, float2 kn) {
   const float2 one = vsplat<float2>(1.0f);
   const float2 ca = vfma(vsplat<float2>(0.17f), kn_power(kn), one);
   const float2 num = vmul(vmul(inv_k, ca), vadd(one, kn));
   const float2 den = vmul(vfma(vsplat<float2>(1.358f), kn, ca), vfma(vsplat<float2>(5.0f), kn, one));
   return div_newton(num, den);
+}
+__device__ __forceinline__ float2 dynamic_inv_k(float2 inv_k, float2 drho_s, float2 kn0,
+                                                const StepArgs &a) {
+  const float2 kn = dynamic_kn(drho_s, kn0, a);
+  if (!kn_common(kn, a))  // the one-node form, lane by lane
+    return make_float2(inv_ka_dynamic(inv_k.x, kn.x, a.kn_model),
+                       inv_ka_dynamic(inv_k.y, kn.y, a.kn_model));
+  return inv_ka_common(inv_k, kn);
+}
+
+// Moments of Eq. 16a (drho_s, mx, my, rho of s); returns 1 / (S rho).
+// SCALED = false: S = 1 (FP32 storage), whose products are left out.
+template <bool SCALED = true, class V>
+__device__ __forceinline__ V node_moments(const V d[9], const StepArgs &a, NodeStateT<V> &s) {
+  s.drho_s = vadd(vadd(vadd(d[0], vadd(d[1], d[3])), vadd(d[2], d[4])),
+                  vadd(vadd(d[5], d[7]), vadd(d[6], d[8])));
+  // sum_i w_i e_i = 0, so the momentum of the deviations is the momentum.
+  const V d57 = vsub(d[5], d[7]), d86 = vsub(d[8], d[6]);
+  s.mx = vadd(vsub(d[1], d[3]), vadd(d57, d86));
+  s.my = vadd(vsub(d[2], d[4]), vsub(d57, d86));
+  if (!SCALED) {
+    s.rho = vadd(s.drho_s, vsplat<V>(a.rho0));
+    return vrcp(s.rho);
+  }
+  s.rho = vfma(s.drho_s, vsplat<V>(a.inv_scale), vsplat<V>(a.rho0));
+  return vmul(vsplat<V>(a.inv_scale), vrcp(s.rho));
 }
 
 // Moments of Eq. 16a and the state of a node (one node, or a pair of nodes
@@ -413,14 +443,7 @@ __device__ __forceinline__ NodeStateT<V> node_state_t(const V d[9], V eps, V inv
                                                       const StepArgs &a,
                                                       V kn0 = vsplat<V>(0.0f)) {
   NodeStateT<V> s;
-  s.drho_s = vadd(vadd(vadd(d[0], vadd(d[1], d[3])), vadd(d[2], d[4])),
-                  vadd(vadd(d[5], d[7]), vadd(d[6], d[8])));
-  // sum_i w_i e_i = 0, so the momentum of the deviations is the momentum.
-  const V d57 = vsub(d[5], d[7]);
-  s.mx = vadd(vsub(d[1], d[3]), vadd(d57, vsub(d[8], d[6])));
-  s.my = vadd(vsub(d[2], d[4]), vadd(d57, vsub(d[6], d[8])));
-  s.rho = vfma(s.drho_s, vsplat<V>(a.inv_scale), vsplat<V>(a.rho0));
-  const V c = vmul(vsplat<V>(a.inv_scale), vrcp(s.rho));  // 1 / (S rho)
+  const V c = node_moments(d, a, s);
   if constexpr (sizeof(V) == sizeof(float)) {
     if (eps > 0.0f) {
       if (DYN) inv_k = dynamic_inv_k(inv_k, s.drho_s, kn0, a);
@@ -487,12 +510,13 @@ __device__ __forceinline__ V wmul(float wh, float wl, V t) {
 // rounding (zero-mean with stochastic rounding) dominates their effect.
 template <bool HILO, class V>
 __device__ __forceinline__ void collide_t(V d[9], const NodeStateT<V> &s, const StepArgs &a) {
-  const V rs = vmul(s.rho, vsplat<V>(a.scale));
+  const V rs = HILO ? s.rho : vmul(s.rho, vsplat<V>(a.scale));  // HILO: FP32 storage, S = 1
   const V ux = s.ux, uy = s.uy, Fx = s.Fx, Fy = s.Fy, ie = s.ieps;
-  const V om = vsplat<V>(a.omega), cf = vsplat<V>(a.cforce);
+  const V om = vsplat<V>(a.omega);
   const V usq = vmul(vmul(vsplat<V>(1.5f), ie), vfma(ux, ux, vmul(uy, uy)));
   const V uF3 = vmul(vmul(vsplat<V>(3.0f), ie), vfma(ux, Fx, vmul(uy, Fy)));
-  const V A = vfma(om, s.drho_s, vneg(vmul(rs, vfma(om, usq, vmul(cf, uF3)))));
+  const V mom = vsplat<V>(-a.omega), mcf = vsplat<V>(-a.cforce);
+  const V A = vfma(om, s.drho_s, vmul(rs, vfma(mom, usq, vmul(mcf, uF3))));
   // P = 3 (X, Y); every sum with a product below is one fma
   const V X = vfma(om, s.mx, s.rFx), Y = vfma(om, s.my, s.rFy);
   const V three = vsplat<V>(3.0f), mthree = vsplat<V>(-3.0f);
@@ -504,7 +528,7 @@ __device__ __forceinline__ void collide_t(V d[9], const NodeStateT<V> &s, const 
   const V sx = vfma(ux, tx, A), sy = vfma(uy, ty, A), sd = vfma(uy, ty, sx);
   const V s5 = vadd(sd, Mxy2), s6 = vsub(sd, Mxy2);
   const V Py = vmul(three, Y);
-  const V pp = vfma(three, X, Py), pm = vfma(three, X, vneg(Py));
+  const V pp = vfma(three, X, Py), pm = vfma(mthree, X, Py);  // P_x + P_y, P_y - P_x
   const V o1 = vsplat<V>(a.one_m_omega);
   d[0] = vfma(o1, d[0], wmul<HILO>(kW0h, kW0l, A));
   d[1] = vfma(o1, d[1], wmul<HILO>(kW1h, kW1l, vfma(three, X, sx)));
@@ -513,8 +537,8 @@ __device__ __forceinline__ void collide_t(V d[9], const NodeStateT<V> &s, const 
   d[4] = vfma(o1, d[4], wmul<HILO>(kW1h, kW1l, vfma(mthree, Y, sy)));
   d[5] = vfma(o1, d[5], wmul<HILO>(kW2h, kW2l, vadd(s5, pp)));
   d[7] = vfma(o1, d[7], wmul<HILO>(kW2h, kW2l, vsub(s5, pp)));
-  d[6] = vfma(o1, d[6], wmul<HILO>(kW2h, kW2l, vsub(s6, pm)));
-  d[8] = vfma(o1, d[8], wmul<HILO>(kW2h, kW2l, vadd(s6, pm)));
+  d[6] = vfma(o1, d[6], wmul<HILO>(kW2h, kW2l, vadd(s6, pm)));
+  d[8] = vfma(o1, d[8], wmul<HILO>(kW2h, kW2l, vsub(s6, pm)));
 }
 
 template <bool HILO = true>

@@ -53,7 +53,7 @@ lbmp_status cuda_fail(cudaError_t e, const char *what) {
     if (e_ != cudaSuccess) return cuda_fail(e_, #call);      \
   } while (0)
 
-constexpr int kGraphLevels = 6;   // step graphs of 1, 2, 4, ..., 32 steps
+constexpr int kGraphLevels = 6;   // step graphs of 1, 2, 4, ..., 32 launches
 constexpr uint64_t kStateMagic = 0x4c424d5053544131ull;  // "LBMPSTA1"
 
 struct StateHeader {
@@ -92,6 +92,11 @@ void free_graphs(lbmp_ctx *c) {
         cudaGraphExecDestroy(g);
         g = nullptr;
       }
+  for (auto &g : c->odd)
+    if (g) {
+      cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
 }
 
 void release(lbmp_ctx *c) {
@@ -175,26 +180,26 @@ cudaError_t launch_one(lbmp_ctx *c, const StepArgs &a0, const void *fin, void *f
   return lbmp::launch_step(c->p.storage, c->sr, a, c->rows(), fin, fout, c->med, c->d_tctr, k, s);
 }
 
-// Graph of 2^level steps starting from buffer `cur` (captured once per
-// medium: the launch arguments hold the storage scale), plus the counter
-// bump when the rounding is stochastic.  A replay saves the launch gaps of
-// single launches (~3 us per step at 4096^2).
-lbmp_status get_graph(lbmp_ctx *c, int level, int cur, cudaGraphExec_t *out) {
-  if (c->graph[level][cur]) {
-    *out = c->graph[level][cur];
-    return LBMP_OK;
-  }
-  const int nsteps = 1 << level;
+// Graph of `launches` launches starting from buffer `cur` (captured once
+// per medium: the launch arguments hold the storage scale), each of two steps
+// or of one, plus the counter bump when the rounding is stochastic.  A replay
+// saves the launch gaps of single launches (~3 us per step at 4096^2).
+lbmp_status get_graph(lbmp_ctx *c, cudaGraphExec_t *slot, int launches, bool two, int cur) {
+  if (*slot) return LBMP_OK;
   StepArgs a = c->args();
   cudaGraph_t g = nullptr;
   LBMP_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int b = cur;
+  const int per = two ? 2 : 1;
   cudaError_t err = cudaSuccess;
-  for (int t = 0; t < nsteps && err == cudaSuccess; ++t) {
-    err = launch_one(c, a, c->buf[b], c->buf[b ^ 1], t, c->cap_stream);
+  for (int t = 0; t < launches && err == cudaSuccess; ++t) {
+    err = two ? lbmp::launch_fused(c->p.storage, c->sr, a, c->rows(), c->buf[b], c->buf[b ^ 1],
+                                   c->med, c->d_tctr, t * per, c->nsm, c->cap_stream)
+              : launch_one(c, a, c->buf[b], c->buf[b ^ 1], t, c->cap_stream);
     b ^= 1;
   }
-  if (err == cudaSuccess && c->sr) err = lbmp::launch_bump(c->d_tctr, nsteps, c->cap_stream);
+  if (err == cudaSuccess && c->sr)
+    err = lbmp::launch_bump(c->d_tctr, launches * per, c->cap_stream);
   cudaError_t end = cudaStreamEndCapture(c->cap_stream, &g);
   if (err != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -205,8 +210,7 @@ lbmp_status get_graph(lbmp_ctx *c, int level, int cur, cudaGraphExec_t *out) {
   cudaError_t ie = cudaGraphInstantiate(&exec, g, 0);
   cudaGraphDestroy(g);
   if (ie != cudaSuccess) return cuda_fail(ie, "cudaGraphInstantiate");
-  c->graph[level][cur] = exec;
-  *out = exec;
+  *slot = exec;
   return LBMP_OK;
 }
 
@@ -362,6 +366,8 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     c->staged = p.kernel == LBMP_KERNEL_STAGED ||
                 (p.kernel == LBMP_KERNEL_AUTO && p.storage == LBMP_STORE_FP16);
     c->wide = p.kernel == LBMP_KERNEL_WIDE;
+    c->fused = p.kernel == LBMP_KERNEL_AUTO && c->drop_tile < 0 &&
+               lbmp::fused_covers(p.storage, p.kn_beta != 0.0, p.nx, p.ny);
     e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) {
       delete c;
@@ -556,21 +562,29 @@ lbmp_status lbmp_step(lbmp_ctx *c, int64_t n) {
     const DeviceScope device_scope(c->device);
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
-    // n = 32 q + sum of binary digits: q replays of the 32-step graph, then
-    // one replay of each smaller power of two
-    int64_t left = n;
+    // launches of two steps (or one): q replays of the 32-launch graph, then
+    // one replay of each smaller power of two; an odd step at the end
+    int64_t left = c->fused ? n / 2 : n;
     for (int level = kGraphLevels - 1; level >= 0 && left > 0; --level) {
       const int64_t size = 1ll << level;
       while (left >= size) {
-        cudaGraphExec_t g = nullptr;
-        st = get_graph(c, level, c->cur, &g);
+        cudaGraphExec_t *slot = &c->graph[level][c->cur];
+        st = get_graph(c, slot, (int)size, c->fused, c->cur);
         if (st) return st;
-        LBMP_CK(cudaGraphLaunch(g, c->stream));
+        LBMP_CK(cudaGraphLaunch(*slot, c->stream));
         c->launches += size + (c->sr ? 1 : 0);
         if (size & 1) c->cur ^= 1;  // an odd replay swaps the buffers
         left -= size;
         if (level < kGraphLevels - 1) break;  // one replay of each smaller size
       }
+    }
+    if (c->fused && (n & 1)) {
+      cudaGraphExec_t *slot = &c->odd[c->cur];
+      st = get_graph(c, slot, 1, false, c->cur);
+      if (st) return st;
+      LBMP_CK(cudaGraphLaunch(*slot, c->stream));
+      c->launches += 1 + (c->sr ? 1 : 0);
+      c->cur ^= 1;
     }
     c->steps += n;
     return LBMP_OK;
