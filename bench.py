@@ -752,7 +752,8 @@ def batch_roofline(r, K, peak, kind, storage):
     when they were taken on the current batched-kernel sources and on the
     same set of instances (the same node count)."""
     from paper_1411_7051_gb300 import build as lbuild
-    per_launch_s = r["ms"] * 1e-3 / K
+    spl = steps_per_launch(r.get("launches", K), K)
+    per_launch_s = r["ms"] * 1e-3 / K * spl
     achieved = r["bpu"] * r["nodes"] / per_launch_s / 1e9
     tr = None
     if r["staged"]:
@@ -762,11 +763,13 @@ def batch_roofline(r, K, peak, kind, storage):
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_kind": f"of {kind}",
             "frac_of_nominal": achieved / NOMINAL_HBM_GBS, "nominal_peak": NOMINAL_HBM_GBS,
-            "bytes_per_update": r["bpu"],
+            "bytes_per_update": r["bpu"] / spl, "steps_per_launch": spl,
             "traffic": (tr["dram_bytes_per_launch"] if tr else None),
-            "traffic_per_update": (tr["dram_bytes_per_launch"] / r["nodes"] if tr else None),
+            "traffic_per_update": (tr["dram_bytes_per_launch"] / r["nodes"] / spl
+                                   if tr else None),
             "achieved_dram": (tr["dram_bytes_per_launch"] / per_launch_s / 1e9 if tr else None),
-            "kernel": ("lbmp::batch_staged_kernel" if r["staged"] else "lbmp::batch_step_kernel")}
+            "kernel": ("lbmp::batch_fused_kernel" if spl == 2 else "lbmp::batch_staged_kernel"
+                       if r["staged"] else "lbmp::batch_step_kernel")}
 
 
 def batch_object(lbmp, torch, args):

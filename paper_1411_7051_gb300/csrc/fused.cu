@@ -8,42 +8,35 @@
 
 namespace lbmp {
 
-// Strips and segments of a launch: one warp per strip and segment.  A warp's
-// time is that of its seg + 2 rows (the two halo rows run the first level
-// only), so small segments cost redundant rows and large ones leave the last
-// wave uneven.  w waves of resident warps cost about 0.7 + w / 2 up to one (a
-// partly filled chip runs each row faster), 2.2 up to two, w + 0.25 beyond:
-// fitted to sweeps of seg at 512^2 .. 4096^2, where the choice is within 3% of
-// the best seg measured (1024^2: 6 rows 10.2 us a step, 5 rows 11.8; 4096^2
-// FP32: 28 rows 108.5, one wave of 82 rows 121).
 struct FusedPlan {
-  int strips, seg, tasks;
+  FusedStrips f;
+  int seg, edges, tasks;  // rows per segment; edge warps, all warps
 };
 template <class C>
 static FusedPlan fused_plan(int nx, int rows, int nsm) {
   const double cap = (double)nsm * C::kBlocks * kFusedWarps;
-  const int strips = fused_interior_strips<C>(nx) + 1;
-  const int most = (int)std::max(1.0, std::min((double)rows, 8.0 * cap / strips));
-  FusedPlan best{strips, rows, strips};
+  FusedPlan best{fused_strips<C>(nx), rows, 0, 0};
+  const int most = (int)std::max(1.0, std::min((double)rows, 8.0 * cap / (best.f.inner + 1)));
   double best_cost = -1.0;
   for (int parts = 1; parts <= most; ++parts) {
     const int seg = (rows + parts - 1) / parts;
-    const int tasks = strips * ((rows + seg - 1) / seg);
-    const double w = tasks / cap;
-    const double cost = (seg + 2) * (w <= 1.0 ? 0.7 + 0.5 * w : (w <= 2.0 ? 2.2 : w + 0.25));
+    const int n = (rows + seg - 1) / seg;
+    const int edges = (n + best.f.per - 1) / best.f.per;
+    const int tasks = edges + best.f.inner * n;
+    const double cost = fused_cost(seg, tasks / cap);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
-      best = {strips, seg, tasks};
+      best = {best.f, seg, edges, tasks};
     }
   }
   return best;
 }
 
 // Where two steps per launch are the faster form.  FP16 storage: everywhere
-// (against the staged kernel 64 x 33: 9.8 -> 2.4 us a step, 512^2 6.4 -> 4.9,
-// 4096^2 112.5 -> 105).  FP32: the direct kernel needs fewer rows in a row on
+// (against the staged kernel 64 x 33: 9.8 -> 2.4 us a step, 512^2 6.4 -> 4.7,
+// 4096^2 112.5 -> 97).  FP32: the direct kernel needs fewer rows in a row on
 // small lattices (512^2: 4.5 us against 4.7; 768^2: 7.6 against 7.2; 4096^2: 190
-// against 109), with a dynamic Kn up to about 10^6 nodes (768^2: 8.8 against 10.0;
+// against 113), with a dynamic Kn up to about 10^6 nodes (768^2: 8.8 against 10.0;
 // 1024^2: 13.5 against 11.8).
 bool fused_covers(int storage, bool dyn, int nx, int ny) {
   if (nx < FusedCfg<StoreF32, 1, false>::kCols || ny < kFusedMinNy) return false;
@@ -62,7 +55,7 @@ static cudaError_t launch_fused_q(const StepArgs &a, int rows, const void *fin, 
   fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>
       <<<(plan.tasks + kFusedWarps - 1) / kFusedWarps, kFusedWarps * 32, C::kSmemBytes, s>>>(
           a, (const typename S::T *)fin, (typename S::T *)fout, med, tctr, k, rows, plan.seg,
-          plan.strips, plan.tasks, mom1, mom2);
+          plan.f, plan.edges, plan.tasks, mom1, mom2);
   return cudaGetLastError();
 }
 

@@ -10,12 +10,18 @@
 // once, those with e_y = 0 wait one row and those with e_y = +1 two rows, in
 // registers, already shifted in x.  No shared memory, no barrier, no wait on
 // another warp: warps recompute the two columns at each side of their strip
-// (64 loaded, 60 stored) and two rows per segment.
+// (64 loaded, 60 stored; 128 and 124 with two pairs per lane) and two rows per
+// segment.
 //
-// The columns that an interior strip cannot produce -- the first two and
-// the last two or three of a row, with the periodic wrap or the pressure
-// extrapolation -- belong to one more warp per segment, which runs the same
-// walk with one node per lane over columns nx - 16 .. nx - 1, 0 .. 15.
+// The columns that an interior strip cannot produce -- the first and the
+// last ones of a row, with the periodic wrap or the pressure extrapolation --
+// belong to edge warps, which run the same walk over the last and the first 16
+// (or 8) columns of a row, for two (four) segments at a time: a node pair per
+// lane where nx is even, one node (half the segments) where it is odd.
+//
+// Bound: FP32 by HBM (40 B an update, 4096^2: 190 us a step with one step per
+// pass, 110 - 114 now, 0.87 of the copy bandwidth), FP16 by the issue of some
+// 265 instructions a pair and step (112.5 -> 97 us).
 //
 // Every node is updated with the operations of the single-step kernels, in
 // their order and with their stochastic-rounding bits, so the populations
@@ -24,6 +30,8 @@
 
 #include <cuda_fp16.h>
 #include <stdint.h>
+
+#include <cmath>
 
 #include "lattice.cuh"
 #include "staged.cuh"
@@ -34,16 +42,21 @@ constexpr int kFusedWarps = 4;     // warps (strips) per block
 constexpr int kFusedMinNy = 6;     // a segment and its halo rows stay apart under the wrap
 
 // Configuration of the interior strips: Q node pairs per lane, so a strip
-// loads 64 Q columns and stores those of lanes 1 .. 30.  Each lane copies its
+// loads 64 Q columns and stores all but two at each side.  Each lane copies its
 // own columns of the rows ahead into its part of a shared-memory FIFO
 // (cp.async), kStages - 1 rows ahead of the row in use; the medium stays one
 // row longer, for the second level.
 template <class S, int Q, bool DYN>
 struct FusedCfg {
   using T = typename S::T;
-  static constexpr int kCols = 64 * Q, kHalo = 2 * Q;
-  static constexpr int kOut = 60 * Q;             // from one strip to the next
-  static constexpr int kBlocks = Q == 1 ? 5 : 3;  // resident blocks per SM
+  static constexpr int kCols = 64 * Q;
+  // Columns a strip stores: all but two at each side, or for FP32 with two
+  // pairs per lane those of lanes 1 .. 30, whose rows start on 32-byte sectors
+  // (4096^2: 110 - 114 us a step against 118 with 124 columns).
+  static constexpr int kOut = sizeof(T) == 4 && Q == 2 ? 120 : kCols - 4;
+  static constexpr int kLead = (kCols - kOut) / 2;
+  static constexpr int kAlign = sizeof(T) == 4 && Q == 2 ? 8 : 4;  // of first columns
+  static constexpr int kBlocks = Q == 1 ? 4 : 3;  // resident blocks per SM
   static constexpr int kStages = Q == 1 ? 3 : 2;
   static constexpr int kMedSlots = kStages + 1;
   static constexpr int kPlaneBytes = kCols * (int)sizeof(T);
@@ -71,6 +84,29 @@ __device__ __forceinline__ void copy_wait() {
   asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
+// Stores to global memory: the batched kernel reads its buffer pointers from
+// memory, where the compiler cannot see their address space.
+__device__ __forceinline__ void put_global(float *p, float v) {
+  asm volatile("st.global.f32 [%0], %1;" ::"l"(p), "f"(v) : "memory");
+}
+__device__ __forceinline__ void put_global(float *p, float2 v) {
+  asm volatile("st.global.v2.f32 [%0], {%1, %2};" ::"l"(p), "f"(v.x), "f"(v.y) : "memory");
+}
+__device__ __forceinline__ void put_global(float *p, float2 a, float2 b) {
+  asm volatile("st.global.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(b.x),
+               "f"(b.y)
+               : "memory");
+}
+__device__ __forceinline__ void put_global(__half *p, uint32_t v) {
+  asm volatile("st.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void put_global(__half *p, uint32_t a, uint32_t b) {
+  asm volatile("st.global.v2.u32 [%0], {%1, %2};" ::"l"(p), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ void put_global(__half *p, unsigned short v) {
+  asm volatile("st.global.u16 [%0], %1;" ::"l"(p), "h"(v) : "memory");
+}
+
 // What a lane holds of one direction, in the precision of the storage: the
 // node pair (x, x + 1) for V = float2, one node for V = float.
 template <class S, class V>
@@ -91,9 +127,7 @@ struct LaneRaw<StoreF32, float2> {
   static __device__ __forceinline__ float2 value(R v) { return v; }
   template <bool SR>
   static __device__ __forceinline__ R round(float2 v, uint32_t, int) { return v; }
-  static __device__ __forceinline__ void store(float *p, R v) {
-    *reinterpret_cast<float2 *>(p) = v;
-  }
+  static __device__ __forceinline__ void store(float *p, R v) { put_global(p, v); }
 };
 
 template <>
@@ -107,7 +141,7 @@ struct LaneRaw<StoreF32, float> {
   static __device__ __forceinline__ float value(R v) { return v; }
   template <bool SR>
   static __device__ __forceinline__ R round(float v, uint32_t, int) { return v; }
-  static __device__ __forceinline__ void store(float *p, R v) { *p = v; }
+  static __device__ __forceinline__ void store(float *p, R v) { put_global(p, v); }
 };
 
 template <>
@@ -138,7 +172,7 @@ struct LaneRaw<StoreF16, float2> {
     return packed;
   }
   static __device__ __forceinline__ void store(__half *p, R v) {
-    *reinterpret_cast<uint32_t *>(p) = v;
+    put_global(p, v);
   }
 };
 
@@ -167,7 +201,7 @@ struct LaneRaw<StoreF16, float> {
     return __half_as_ushort(__float2half_rn(v));
   }
   static __device__ __forceinline__ void store(__half *p, R v) {
-    *reinterpret_cast<unsigned short *>(p) = (unsigned short)v;
+    put_global(p, (unsigned short)v);
   }
 };
 
@@ -193,14 +227,32 @@ __device__ __forceinline__ void load_med(const StepArgs &a, const float2 *__rest
   m.kn0 = DYN ? __ldg(a.kn0 + j) : 0.0f;
 }
 
-// Moments and state of the lane's node(s) from the pulled values d.  With
-// one node per lane the pressure columns take their populations from the
-// neighbouring lane first (non-equilibrium extrapolation, as
-// column_from_neighbour).
+// Moments and state of the node(s) of an edge lane from the pulled values d.
+// The pressure columns take their populations from the interior neighbour
+// first (non-equilibrium extrapolation): the other node of the pair, or with
+// one node per lane the neighbouring lane's.
 template <bool DYN>
 __device__ __forceinline__ NodeStateT<float2> lane_state(float2 d[9], const LaneMed<float2> &m,
-                                                         const StepArgs &a, int) {
-  return node_state_t<float2, DYN>(d, m.eps, m.inv_k, a, m.kn0);
+                                                         const StepArgs &a, int x) {
+  NodeStateT<float2> s = node_state_t<float2, DYN>(d, m.eps, m.inv_k, a, m.kn0);
+  if (!a.pressure) return s;
+  const bool lo = x == 0, hi = x + 2 == a.nx;
+  if (lo || hi) {
+    float dn[9], db[9];
+    NodeState sn;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) dn[i] = lo ? d[i].y : d[i].x;
+    sn.drho_s = lo ? s.drho_s.y : s.drho_s.x;
+    sn.rho = lo ? s.rho.y : s.rho.x;
+    sn.ux = lo ? s.ux.y : s.ux.x;
+    sn.uy = lo ? s.uy.y : s.uy.x;
+    column_from_neighbour(a, dn, sn, lo ? m.eps.y : m.eps.x, lo ? 0 : a.nx - 1,
+                          lo ? m.eps.x : m.eps.y, db);
+#pragma unroll
+    for (int i = 0; i < 9; ++i) d[i] = lo ? make_float2(db[i], dn[i]) : make_float2(dn[i], db[i]);
+    s = node_state_t<float2, DYN>(d, m.eps, m.inv_k, a, m.kn0);
+  }
+  return s;
 }
 template <bool DYN>
 __device__ __forceinline__ NodeState lane_state(float d[9], const LaneMed<float> &m,
@@ -252,35 +304,50 @@ __device__ __forceinline__ void lane_collide(V d[9], const NodeStateT<V> &s, con
     p[i] = L::template round<SR>(d[i], SR ? pair_bits(h, i) : 0u, (int)(o & 1));
 }
 
-// The walk of one warp: rows [s0, s1) of level t + 2 over the lane's
-// column(s) x (the pair x, x + 1 for V = float2; x even).  Fluid rows are
-// [a.y0, y_end); with walls those are 1 .. ny - 2.  out: this lane stores.
-// MOM: the moments of levels t and t + 1 go to mom1 and mom2.
+// The walk of the edge warp: the same two levels for groups of lanes, each of
+// which covers the last and the first win / 2 columns of the rows of its own
+// segment (win = 16 or 32; of the window all columns but two at each end come
+// out right), with a node pair per lane (V = float2, nx even) or one node.
+// Rows [s0, s1) are the group's segment, seg >= s1 - s0 the rows every group
+// walks: conditions on rows are per lane, and rows outside the segment and its
+// halo are computed on clamped addresses and not used.  x_lo, x_hi: columns
+// below x_lo or from x_hi on are stored.  MOM: the moments of levels t and t + 1
+// go to mom1 and mom2.
 template <class S, bool SR, bool DYN, bool MOM, class V>
-__device__ __forceinline__ void fused_walk(const StepArgs &a, const typename S::T *__restrict__ fin,
-                                           typename S::T *__restrict__ fout,
-                                           const float2 *__restrict__ med, int x, bool out, int s0,
-                                           int s1, int y_end, uint32_t ts1, uint32_t ts2,
-                                           float *__restrict__ mom1, float *__restrict__ mom2) {
+__device__ __forceinline__ void fused_edges(const StepArgs &a, const typename S::T *__restrict__ fin,
+                                            typename S::T *__restrict__ fout,
+                                            const float2 *__restrict__ med, int win, int x_lo,
+                                            int x_hi, int s0, int s1, int seg, int y_end,
+                                            uint32_t ts1, uint32_t ts2, float *__restrict__ mom1,
+                                            float *__restrict__ mom2) {
   using L = LaneRaw<S, V>;
   using R = typename L::R;
   using T = typename S::T;
+  constexpr int kNodes = (int)(sizeof(V) / sizeof(float));  // per lane
   const long long P = a.plane;
+  const int c = ((threadIdx.x * kNodes) & (win - 1)) - win / 2;  // column, from the row's end on
+  const int x = c < 0 ? a.nx + c : c;
+  const bool out = x < x_lo || x >= x_hi;
   auto wrap = [&](int y) { return y < 0 ? y + a.ny : (y >= a.ny ? y - a.ny : y); };
+  // the row whose first level is computed in the place of row r
+  auto row_of = [&](int r) {
+    r = r < s1 ? r : s1;
+    if (a.walls) r = r < a.y0 ? a.y0 : (r < y_end ? r : y_end - 1);
+    return wrap(r);
+  };
   R raw[9];
   LaneMed<V> m;
-  // Sources of row r.  At a plate the directions that would come from it
+  // Sources of a row.  At a plate the directions that would come from it
   // are the node's own opposite ones, unshifted: planes 4, 7, 8 in the
   // place of 2, 5, 6 (two planes up), or the reverse.
-  auto load_row = [&](int r) {
-    const int y = wrap(r);
-    const T *c = fin + (long long)y * a.pitch + x;
-    const T *u = (a.walls && y == a.y0) ? c + 2 * P : fin + (long long)wrap(r - 1) * a.pitch + x;
-    const T *d = (a.walls && y == y_end - 1) ? c - 2 * P
-                                             : fin + (long long)wrap(r + 1) * a.pitch + x;
-    raw[0] = L::load(c);
-    raw[1] = L::load(c + P);
-    raw[3] = L::load(c + 3 * P);
+  auto load_row = [&](int y) {
+    const T *e = fin + (long long)y * a.pitch + x;
+    const T *u = (a.walls && y == a.y0) ? e + 2 * P : fin + (long long)wrap(y - 1) * a.pitch + x;
+    const T *d = (a.walls && y == y_end - 1) ? e - 2 * P
+                                             : fin + (long long)wrap(y + 1) * a.pitch + x;
+    raw[0] = L::load(e);
+    raw[1] = L::load(e + P);
+    raw[3] = L::load(e + 3 * P);
     raw[2] = L::load(u + 2 * P);
     raw[5] = L::load(u + 5 * P);
     raw[6] = L::load(u + 6 * P);
@@ -289,60 +356,52 @@ __device__ __forceinline__ void fused_walk(const StepArgs &a, const typename S::
     raw[8] = L::load(d + 8 * P);
     load_med<DYN>(a, med, (long long)y * a.pitch + x, m);
   };
-  // first level: rows s0 - 1 .. s1, without the plates
-  const int r0 = a.walls && s0 == a.y0 ? s0 : s0 - 1;
-  const int r_last = a.walls && s1 == y_end ? s1 - 1 : s1;
-  load_row(r0);
+  load_row(row_of(s0 - 1));
   R h0 = R(), h1 = R(), h3 = R();   // e_y = 0 of row r - 1, shifted
   R b2 = R(), b5 = R(), b6 = R();   // e_y = +1 of row r - 2, shifted
   R c2 = R(), c5 = R(), c6 = R();   // e_y = +1 of row r - 1, shifted
-  LaneMed<V> m1 = m;                // medium of row r - 1
+  LaneMed<V> m1 = m;            // medium of row r - 1
 #pragma unroll 1
-  for (int r = r0; r <= s1; ++r) {
+  for (int n = 0; n <= seg + 1; ++n) {
+    const int r = s0 - 1 + n, y = row_of(r);
+    const LaneMed<V> m0 = m;
+    V d[9];
     R p[9];
-    R f4, f7, f8;                   // e_y = -1 of row r, shifted
-    LaneMed<V> m0 = m;
-    if (r <= r_last) {
-      const int y = wrap(r);
-      V d[9];
-      d[0] = L::value(raw[0]);
-      d[2] = L::value(raw[2]);
-      d[4] = L::value(raw[4]);
-      d[1] = L::value(L::from_left(raw[1]));
-      d[3] = L::value(L::from_right(raw[3]));
-      R t5 = L::from_left(raw[5]), t6 = L::from_right(raw[6]);
-      R t7 = L::from_right(raw[7]), t8 = L::from_left(raw[8]);
-      if (a.walls) {
-        if (y == a.y0) {
-          t5 = raw[5];
-          t6 = raw[6];
-        }
-        if (y == y_end - 1) {
-          t7 = raw[7];
-          t8 = raw[8];
-        }
-      }
-      d[5] = L::value(t5);
-      d[6] = L::value(t6);
-      d[7] = L::value(t7);
-      d[8] = L::value(t8);
-      if (r < r_last) load_row(r + 1);
+    R t5 = L::from_left(raw[5]), t6 = L::from_right(raw[6]);
+    R t7 = L::from_right(raw[7]), t8 = L::from_left(raw[8]);
+    d[0] = L::value(raw[0]);
+    d[2] = L::value(raw[2]);
+    d[4] = L::value(raw[4]);
+    d[1] = L::value(L::from_left(raw[1]));
+    d[3] = L::value(L::from_right(raw[3]));
+    if (a.walls && y == a.y0) {
+      t5 = raw[5];
+      t6 = raw[6];
+    }
+    if (a.walls && y == y_end - 1) {
+      t7 = raw[7];
+      t8 = raw[8];
+    }
+    d[5] = L::value(t5);
+    d[6] = L::value(t6);
+    d[7] = L::value(t7);
+    d[8] = L::value(t8);
+    if (n <= seg) load_row(row_of(r + 1));
+    {
       const NodeStateT<V> s = lane_state<DYN>(d, m0, a, x);
       const long long o = (long long)y * a.pitch + x;
       if (MOM && out && r >= s0 && r < s1) store_moments(mom1 + o, P, s);
       lane_collide<S, SR>(d, s, a, o, ts1, p);
-      f4 = p[4];
-      f7 = L::from_right(p[7]);
-      f8 = L::from_left(p[8]);
-    } else {
-      // row r is a plate: row r - 1 gets its own e_y = +1 values back
-      f4 = c2;
-      f7 = L::from_right(c5);  // undoes the shift of c5 (from the left)
-      f8 = L::from_left(c6);
     }
-    if (r > s0) {
-      // second level at row r - 1 (inside the segment: no wrap)
-      V d[9];
+    R f4 = p[4], f7 = L::from_right(p[7]), f8 = L::from_left(p[8]);  // e_y = -1 of row r
+    // beyond the last row below a plate: that row's own e_y = +1 values
+    const R g7 = L::from_right(c5), g8 = L::from_left(c6);  // undo the shifts
+    if (a.walls && r == y_end) {
+      f4 = c2;
+      f7 = g7;
+      f8 = g8;
+    }
+    if (n >= 2) {  // second level at row r - 1
       d[0] = L::value(h0);
       d[1] = L::value(h1);
       d[3] = L::value(h3);
@@ -356,27 +415,25 @@ __device__ __forceinline__ void fused_walk(const StepArgs &a, const typename S::
       const long long o = (long long)(r - 1) * a.pitch + x;
       R q[9];
       lane_collide<S, SR>(d, s, a, o, ts2, q);
-      if (out) {
+      if (out && r - 1 < s1) {
         if (MOM) store_moments(mom2 + o, P, s);
         T *g = fout + o;
 #pragma unroll
         for (int i = 0; i < 9; ++i) L::store(g + i * P, q[i]);
       }
     }
-    if (r <= r_last) {
-      // row a.y0 bounces its e_y = -1 values off the plate below
-      const bool plate = a.walls && r == a.y0;
-      b2 = plate ? p[4] : c2;
-      b5 = plate ? p[7] : c5;
-      b6 = plate ? p[8] : c6;
-      c2 = p[2];
-      c5 = L::from_left(p[5]);
-      c6 = L::from_right(p[6]);
-      h0 = p[0];
-      h1 = L::from_left(p[1]);
-      h3 = L::from_right(p[3]);
-      m1 = m0;
-    }
+    // row a.y0 bounces its e_y = -1 values off the plate below
+    const bool plate = a.walls && r == a.y0;
+    b2 = plate ? p[4] : c2;
+    b5 = plate ? p[7] : c5;
+    b6 = plate ? p[8] : c6;
+    c2 = p[2];
+    c5 = L::from_left(p[5]);
+    c6 = L::from_right(p[6]);
+    h0 = p[0];
+    h1 = L::from_left(p[1]);
+    h3 = L::from_right(p[3]);
+    m1 = m0;
   }
 }
 
@@ -405,16 +462,16 @@ __device__ __forceinline__ void lane_row(const __half *row, int lane, uint32_t v
 template <int Q>
 __device__ __forceinline__ void store_row(float *p, const float2 v[Q]) {
   if constexpr (Q == 2)
-    *reinterpret_cast<float4 *>(p) = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+    put_global(p, v[0], v[1]);
   else
-    *reinterpret_cast<float2 *>(p) = v[0];
+    put_global(p, v[0]);
 }
 template <int Q>
 __device__ __forceinline__ void store_row(__half *p, const uint32_t v[Q]) {
   if constexpr (Q == 2)
-    *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
+    put_global(p, v[0], v[1]);
   else
-    *reinterpret_cast<uint32_t *>(p) = v[0];
+    put_global(p, v[0]);
 }
 
 // Values one column to the left (right) of the lane's pairs.
@@ -460,7 +517,7 @@ __device__ __forceinline__ void copy_row(const R v[Q], R o[Q]) {
 template <class S, bool SR, bool DYN, bool MOM, int Q>
 __device__ __forceinline__ void level_row(typename LaneRaw<S, float2>::R t[9][Q],
                                           const unsigned char *ms, const StepArgs &a,
-                                          long long o, uint32_t ts, bool mom_out,
+                                          long long o, uint32_t ts, bool mom_rows,
                                           float *__restrict__ mom) {
   using L = LaneRaw<S, float2>;
   using C = FusedCfg<S, Q, DYN>;
@@ -497,7 +554,8 @@ __device__ __forceinline__ void level_row(typename LaneRaw<S, float2>::R t[9][Q]
   }
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
-    if (MOM && mom_out) store_moments(mom + o + 2 * q, a.plane, s[q]);
+    if (MOM && mom_rows && (C::kLead == 2 && Q == 2 ? (q == 0 ? lane > 0 : lane < 31) : lane > 0 && lane < 31))
+      store_moments(mom + o + 2 * q, a.plane, s[q]);
     typename L::R p[9];
     lane_collide<S, SR, float2>(d[q], s[q], a, o + 2 * q, ts, p);
 #pragma unroll
@@ -520,6 +578,8 @@ __device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S:
   constexpr int NS = C::kStages, NM = C::kMedSlots;
   const int lane = threadIdx.x & 31;
   const long long P = a.plane;
+  // the kLead columns at each side are not right: those of lanes 0 and 31, or
+  // (kLead = 2 with two pairs a lane) half of theirs
   const bool out = lane >= 1 && lane <= 30;
   const int x = c0 + 2 * Q * lane;
   const int r0 = a.walls && s0 == a.y0 ? s0 : s0 - 1;
@@ -608,7 +668,7 @@ __device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S:
         from_left<Q>(w, t[8]);
       }
       level_row<S, SR, DYN, MOM, Q>(t, m_now, a, (long long)y * a.pitch + x, ts1,
-                                    MOM && out && r >= s0 && r < s1, mom1);
+                                    MOM && r >= s0 && r < s1, mom1);
       copy_row<Q>(t[4], f4);
       from_right<Q>(t[7], f7);
       from_left<Q>(t[8], f8);
@@ -633,11 +693,16 @@ __device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S:
         u[8][q] = f8[q];
       }
       const long long o = (long long)(r - 1) * a.pitch + x;
-      level_row<S, SR, DYN, MOM, Q>(u, m_was, a, o, ts2, MOM && out, mom2);
+      level_row<S, SR, DYN, MOM, Q>(u, m_was, a, o, ts2, MOM, mom2);
+      T *g = fout + o;
       if (out) {
-        T *g = fout + o;
 #pragma unroll
         for (int i = 0; i < 9; ++i) store_row<Q>(g + i * P, u[i]);
+      } else if (C::kLead == 2 && Q == 2) {
+        const int q = lane == 0 ? Q - 1 : 0;
+#pragma unroll
+        for (int i = 0; i < 9; ++i)
+          LaneRaw<S, float2>::store(g + i * P + 2 * q, lane == 0 ? u[i][Q - 1] : u[i][0]);
       }
     }
     if (r <= r_last) {
@@ -662,37 +727,76 @@ __device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S:
   }
 }
 
-// Interior strips of a lattice nx wide: they store columns kHalo .., kOut a
-// strip, the last one moved left to end inside the row (it stores some columns
-// again, with the same values).
+// Strips of a lattice nx wide: `inner` interior ones, the first at column
+// c0 and the others kOut apart (the last one moved left if it would leave the
+// row; it then stores some columns again, with the same values), and the edge
+// warp's columns below x_lo and from x_hi on, in windows of `win` columns.  A
+// window of 16 covers 6 columns at each end of a row, one of 32 covers 14: the
+// wider one where it saves a strip.  An edge warp holds `per` windows, of
+// consecutive segments.
+struct FusedStrips {
+  int inner, c0, last, win, per, x_lo, x_hi;
+};
 template <class C>
-__host__ __device__ inline int fused_last_column(int nx) { return (nx - C::kCols) & ~3; }
-template <class C>
-__host__ __device__ inline int fused_interior_strips(int nx) {
-  return (fused_last_column<C>(nx) + C::kOut - 1) / C::kOut + 1;
+__host__ __device__ inline FusedStrips fused_strips(int nx) {
+  FusedStrips f{};
+  for (int win = 32; win >= 16; win -= 16) {
+    const int edge = win / 2 - 2;
+    const int last = (nx - C::kCols) & ~3;
+    int c0 = (edge - C::kLead) / C::kAlign * C::kAlign;
+    c0 = c0 < last ? c0 : last;
+    const int left = nx - edge - c0 - C::kLead;
+    const int n = left > C::kOut ? (left + C::kOut - 1) / C::kOut : 1;
+    const int end = c0 + (n - 1) * C::kOut < last ? c0 + (n - 1) * C::kOut : last;
+    if (win == 32 || (n <= f.inner && nx - (end + C::kCols - C::kLead) <= edge)) {
+      f = {n, c0, last, win, (nx & 1 ? 32 : 64) / win, c0 + C::kLead, end + C::kCols - C::kLead};
+    }
+  }
+  return f;
 }
 
-// One warp's task: strip `strip` (the last is the edge strip) of rows [s0, s1).
+// Relative time of a launch in segments of seg rows and w waves of resident
+// warps, one warp per strip and segment.  A warp's time is that of its seg + 2
+// rows (the two halo rows run the first level only), so small segments cost
+// redundant rows and large ones leave the last wave uneven: up to one wave
+// 0.7 + w / 2 (a partly filled chip runs each row faster), 2.2 up to two, w + 0.25
+// beyond and a little more where the last wave is nearly empty.  Fitted to
+// sweeps of seg at 512^2 .. 4096^2 (1024^2: 6 rows 10.2 us a step, 5 rows 11.8;
+// 4096^2 FP32: 20 and 28 rows 110.5, 25 rows 113, one wave of 82 rows 121).
+inline double fused_cost(int seg, double w) {
+  if (w <= 1.0) return (seg + 2) * (0.7 + 0.5 * w);
+  if (w <= 2.0) return (seg + 2) * 2.2;
+  return (seg + 2) * (w + 0.25 + 0.15 * (std::ceil(w) - w));
+}
+
+// One warp's task: strip `strip` of the segment that starts at row s0, seg
+// rows high at most; strip < 0: the edges of that segment and the next per - 1.
 template <class S, bool SR, bool DYN, bool MOM, int Q>
 __device__ __forceinline__ void fused_task(const StepArgs &a, const typename S::T *__restrict__ fin,
                                            typename S::T *__restrict__ fout,
-                                           const float2 *__restrict__ med, int strip, int s0,
-                                           int s1, int y_end, uint32_t ts1, uint32_t ts2,
-                                           float *__restrict__ mom1, float *__restrict__ mom2,
-                                           unsigned char *ring) {
+                                           const float2 *__restrict__ med, const FusedStrips &f,
+                                           int strip, int s0, int seg, int y_end, uint32_t ts1,
+                                           uint32_t ts2, float *__restrict__ mom1,
+                                           float *__restrict__ mom2, unsigned char *ring) {
   using C = FusedCfg<S, Q, DYN>;
-  const int lane = threadIdx.x & 31;
-  const int last = fused_last_column<C>(a.nx);
-  if (strip < fused_interior_strips<C>(a.nx)) {
-    const int c0 = strip * C::kOut < last ? strip * C::kOut : last;
+  if (strip >= 0) {
+    const int c0 = f.c0 + strip * C::kOut < f.last ? f.c0 + strip * C::kOut : f.last;
+    const int s1 = s0 + seg < y_end ? s0 + seg : y_end;
     fused_strip<S, SR, DYN, MOM, Q>(a, fin, fout, med, c0, s0, s1, y_end, ts1, ts2, mom1, mom2,
                                     ring);
   } else {
-    // at most kHalo columns on the left and kHalo + 3 on the right
-    const int x = lane < 16 ? a.nx - 16 + lane : lane - 16;
-    const bool out = x < C::kHalo || x >= last + C::kCols - C::kHalo;
-    fused_walk<S, SR, DYN, MOM, float>(a, fin, fout, med, x, out, s0, s1, y_end, ts1, ts2, mom1,
-                                       mom2);
+    s0 += (int)((threadIdx.x & 31) / (32 / f.per)) * seg;
+    // a window past the last row repeats the first segment, without storing
+    const bool none = s0 >= y_end;
+    s0 = none ? a.y0 : s0;
+    const int s1 = s0 + seg < y_end ? s0 + seg : y_end;
+    const int x_lo = none ? 0 : f.x_lo, x_hi = none ? a.nx : f.x_hi;
+    if (a.nx & 1)
+      fused_edges<S, SR, DYN, MOM, float>(a, fin, fout, med, f.win, x_lo, x_hi, s0, s1, seg, y_end,
+                                          ts1, ts2, mom1, mom2);
+    else
+      fused_edges<S, SR, DYN, MOM, float2>(a, fin, fout, med, f.win, x_lo, x_hi, s0, s1, seg, y_end,
+                                           ts1, ts2, mom1, mom2);
   }
 }
 
@@ -701,33 +805,32 @@ __device__ __forceinline__ uint32_t level_hash(const StepArgs &a, unsigned long 
   return mix32((uint32_t)t * 0x9e3779b9u ^ a.seed_lo ^ mix32((uint32_t)(t >> 32) ^ a.seed_hi));
 }
 
-// Task w of the launch: strip w % strips of segment w / strips, the
-// segments being `seg` rows high (the last one shorter).  FORCH = a0.forch, as
-// a constant: no branch inside a row.
+// Task w of the launch: the edge warps first (they take longest per row),
+// then strip by strip of segment after segment, seg rows high (the last one
+// shorter).  FORCH = a0.forch, as a constant: no branch inside a row.
 template <class S, bool SR, bool DYN, bool MOM, bool FORCH, int Q>
 __global__ void __launch_bounds__(kFusedWarps * 32, FusedCfg<S, Q, DYN>::kBlocks)
     fused_step_kernel(const StepArgs a0, const typename S::T *__restrict__ fin,
                       typename S::T *__restrict__ fout, const float2 *__restrict__ med,
                       const unsigned long long *__restrict__ tctr, int k, int rows, int seg,
-                      int strips, int tasks, float *__restrict__ mom1, float *__restrict__ mom2) {
+                      const FusedStrips f, int edges, int tasks, float *__restrict__ mom1,
+                      float *__restrict__ mom2) {
   extern __shared__ __align__(128) unsigned char smem[];
   StepArgs a = a0;
   a.forch = FORCH;
   const int warp = threadIdx.x >> 5;
   const int w = blockIdx.x * kFusedWarps + warp;
   if (w >= tasks) return;
-  const int strip = w % strips, part = w / strips;
-  const int y_end = a.y0 + rows;
-  const int s0 = a.y0 + part * seg;
-  const int s1 = s0 + seg < y_end ? s0 + seg : y_end;
+  const int strip = w < edges ? -1 : (w - edges) % f.inner;
+  const int part = w < edges ? w * f.per : (w - edges) / f.inner;
   uint32_t ts1 = 0, ts2 = 0;
   if (SR) {
     const unsigned long long t = *tctr + (unsigned long long)k;
     ts1 = level_hash(a, t);
     ts2 = level_hash(a, t + 1);
   }
-  fused_task<S, SR, DYN, MOM, Q>(a, fin, fout, med, strip, s0, s1, y_end, ts1, ts2, mom1, mom2,
-                                 smem + warp * FusedCfg<S, Q, DYN>::kWarpBytes);
+  fused_task<S, SR, DYN, MOM, Q>(a, fin, fout, med, f, strip, a.y0 + part * seg, seg, a.y0 + rows,
+                                 ts1, ts2, mom1, mom2, smem + warp * FusedCfg<S, Q, DYN>::kWarpBytes);
 }
 
 }  // namespace lbmp

@@ -68,3 +68,40 @@ def test_permeable_everywhere_and_nowhere():
         case = _case(1024, 520, True, True, 1, 0.0, p_solid)
         _same(case, FP32, DIRECT)
         _same(case, FP16, STAGED)
+
+
+@pytest.mark.parametrize("walls,pressure", [(False, False), (True, True)])
+@pytest.mark.parametrize("storage,rounding", [(FP32, 0), (FP16, 0), (FP16, 1)])
+@pytest.mark.parametrize("sizes", [[(64, 6), (131, 20), (256, 64), (300, 41), (65, 9)],
+                                   [(128, 400), (1024, 513), (1003, 700)]])
+def test_batch_pairs_match_single_steps(sizes, storage, rounding, walls, pressure):
+    """The staged candidate advances a batch two steps per launch; steps asked
+    for one by one run its single-step kernel.  Both give the same bits."""
+    from paper_1411_7051_gb300 import lbmp
+    cfg = lbmp.SimConfig(1, 1, tau=0.75, G=(1e-5, 2e-6), forchheimer=1, storage=storage,
+                         bc_x=lbmp.BCX_PRESSURE if pressure else lbmp.BCX_PERIODIC,
+                         bc_y=lbmp.BCY_WALLS if walls else lbmp.BCY_PERIODIC, rho_in=1.001,
+                         rho_out=0.999, fp16_rounding=rounding, seed=11)
+    out = []
+    for pairs in (True, False):
+        with lbmp.Batch(cfg, sizes) as b:
+            b.set_shape(9)
+            for i, (nx, ny) in enumerate(sizes):
+                m = media.random_medium(nx, ny, seed=i, p_open=0.1, p_solid=0.05,
+                                        log10_k_range=(-3, 0))
+                b.set_fields(i, m.eps, m.k_i, m.kn)
+            launches = b.info().launches
+            for n in (37, 4):   # one graph replay of 32 steps, pairs and a single step
+                if pairs:
+                    b.step(n)
+                else:
+                    for _ in range(n):
+                        b.step(1)
+            b.synchronize()
+            out.append(([b.populations(i) for i in range(len(sizes))], b.permeability()[0],
+                        b.info().launches - launches))
+    (pa, ka, la), (pb, kb, lb) = out
+    assert la < lb
+    for fa, fb in zip(pa, pb):
+        assert bool((fa == fb).all()), f"{int((fa != fb).sum())} populations differ"
+    assert np.array_equal(ka, kb)
