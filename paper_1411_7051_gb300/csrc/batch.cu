@@ -30,6 +30,7 @@
 #include "nvtx_range.h"
 #include "lattice.cuh"
 #include "lbmp.h"
+#include "readout.cuh"
 #include "fused.cuh"
 #include "staged.cuh"
 
@@ -449,74 +450,72 @@ static double batch_fused_capacity(int q, int nsm) {
          (q == 2 ? FusedCfg<StoreF32, 2, false>::kBlocks : FusedCfg<StoreF32, 1, false>::kBlocks);
 }
 
-// Per-instance reductions: block partials over the work list (one 256-node
-// segment per item), then one block per instance sums its items in order.
-constexpr int kBatchMacroBX = 256;
+// Per-instance sums of u_x (and non-finite nodes): an item is 256 columns x
+// `chunk` rows of an instance, one block each, a node's velocity one FP64 add
+// (FP64 runs at ~1/64 of the FP32 rate); then one block per instance adds its
+// items in order.  Six FP64 quantities and a reduction tree per node took
+// 0.81 ms on 11.4 M nodes.
+constexpr int kBatchMaxChunk = 32;
 
 template <class S>
-__global__ void __launch_bounds__(kBatchMacroBX)
-    batch_macro_kernel(const BatchInst *__restrict__ inst, const long long *__restrict__ cum,
-                       int count, int parity, double *__restrict__ partials) {
-  const long long items = cum[count];
-  for (long long w = blockIdx.x; w < items; w += gridDim.x) {
-    const int ii = find_instance(cum, count, w);
-    const BatchInst &I = inst[ii];
-    const StepArgs &a = I.a;
-    const long long local = w - cum[ii];
-    const int xblocks = (a.nx + kBatchMacroBX - 1) / kBatchMacroBX;
-    const int y = a.y0 + (int)(local / xblocks);
-    const int x = (int)(local % xblocks) * kBatchMacroBX + threadIdx.x;
-    const typename S::T *fin = (const typename S::T *)I.buf[parity];
-    double v[kNQ] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-    if (x < a.nx) {
-      float d[9];
-      const float2 m = I.med[(long long)y * a.pitch + x];
-      pull_node<S>(fin, a, x, y, d);
-      if (a.pressure && (x == 0 || x == a.nx - 1)) pressure_node<S>(fin, I.med, a, x, y, m.x, d);
-      const NodeState s = node_state(d, m.x, m.y, a);
-      const bool finite = isfinite(s.ux) && isfinite(s.uy) && isfinite(s.rho);
-      v[0] = finite ? (double)s.ux : 0.0;
-      v[1] = finite ? (double)s.uy : 0.0;
-      v[2] = finite ? (double)(s.drho_s * a.inv_scale) : 0.0;
-      v[3] = finite ? (double)s.ux * s.ux + (double)s.uy * s.uy : 0.0;
-      v[5] = finite ? 0.0 : 1.0;
+__global__ void __launch_bounds__(kReadBX, 3)
+    batch_sums_kernel(const StepArgs base, const BatchInst *__restrict__ inst,
+                      const long long *__restrict__ cum,
+                      int count, int chunk, int parity, double *__restrict__ partials) {
+  const long long w = blockIdx.x;
+  const int ii = find_instance(cum, count, w);
+  const BatchInst &I = inst[ii];
+  StepArgs a = base;
+  a.nx = I.a.nx;
+  a.ny = I.a.ny;
+  a.pitch = I.a.pitch;
+  a.plane = I.a.plane;
+  a.scale = I.a.scale;
+  a.inv_scale = I.a.inv_scale;
+  const int local = (int)(w - cum[ii]);
+  const int xblocks = (a.nx + kReadBX - 1) / kReadBX;
+  const int y0 = a.y0 + (local / xblocks) * chunk;
+  const int y1 = min(y0 + chunk, a.y0 + I.rows);
+  const PairIn<S> p((const typename S::T *)I.buf[parity], I.med, a,
+                    (local % xblocks) * kReadBX + (int)threadIdx.x);
+  Sums v = {0.0, 0.0, 0u};
+  auto add = [&](float ux, float uy, float rho) {
+    if (finite_node(ux, uy, rho))
+      v.a += wide_value(ux);
+    else
+      ++v.bad;
+  };
+  if (p.x < a.nx) {
+#pragma unroll 1
+    for (int y = y0; y < y1; y += 2) {
+      const bool both = y + 1 < y1;
+      typename PairIn<S>::Raw r;
+      p.template load<false>(y, both ? y + 1 : y, r);
+      const NodeStateT<float2> s = p.template state<false>(r);
+      add(s.ux.x, s.uy.x, s.rho.x);
+      if (both) add(s.ux.y, s.uy.y, s.rho.y);
     }
-    __shared__ double red[kBatchMacroBX / 32][kNQ];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int q = 0; q < kNQ; ++q) {
-      double t = v[q];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) t += __shfl_down_sync(0xffffffffu, t, off);
-      if (lane == 0) red[warp][q] = t;
-    }
-    __syncthreads();
-    if (threadIdx.x < kNQ) {
-      double t = 0.0;
-      for (int ww = 0; ww < kBatchMacroBX / 32; ++ww) t += red[ww][threadIdx.x];
-      partials[w * kNQ + threadIdx.x] = t;
-    }
-    __syncthreads();
+  }
+  v = block_sums(v);
+  if (threadIdx.x == 0) {
+    partials[2 * w] = v.a;
+    partials[2 * w + 1] = (double)v.bad;
   }
 }
 
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kReadBX)
     batch_finalize_kernel(const long long *__restrict__ cum, const double *__restrict__ partials,
                           double *__restrict__ out) {
-  __shared__ double sh[256];
   const int ii = blockIdx.x;
-  const long long b0 = cum[ii], b1 = cum[ii + 1];
-  for (int q = 0; q < kNQ; ++q) {
-    double t = 0.0;
-    for (long long b = b0 + threadIdx.x; b < b1; b += 256) t += partials[b * kNQ + q];
-    sh[threadIdx.x] = t;
-    __syncthreads();
-    for (int s = 128; s > 0; s >>= 1) {
-      if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) out[(long long)ii * kNQ + q] = sh[0];
-    __syncthreads();
+  Sums v = {0.0, 0.0, 0u};
+  for (long long b = cum[ii] + threadIdx.x; b < cum[ii + 1]; b += kReadBX) {
+    v.a += partials[2 * b];
+    v.b += partials[2 * b + 1];
+  }
+  v = block_sums(v);
+  if (threadIdx.x == 0) {
+    out[2 * ii] = v.a;
+    out[2 * ii + 1] = v.b;
   }
 }
 
@@ -632,8 +631,9 @@ struct lbmp_batch {
   long long items_cap = 0;           // capacity of d_item_inst
   long long *d_cum_macro = nullptr;  // work list of the reductions
   long long items_step = 0, items_macro = 0;
-  double *d_partials = nullptr;      // [items_macro][kNQ]
-  double *d_results = nullptr;       // [count][kNQ]
+  int sum_chunk = 1;                 // rows of an item of the reductions
+  double *d_partials = nullptr;      // [items_macro][2]
+  double *d_results = nullptr;       // [count][2]
   double *d_med_partials = nullptr;  // set_fields scratch
   double *d_med_results = nullptr;
   unsigned *d_flag = nullptr;
@@ -995,8 +995,16 @@ lbmp_status lbmp_batch_create(const lbmp_params *pin, int32_t count, const int32
       BTRY(balloc(b, &m, (size_t)a.plane * sizeof(float2), "batch medium"));
       I.med = (const float2 *)m;
     }
-    const std::vector<long long> cum_macro = work_list(b, lbmp::kBatchMacroBX);
+    // rows per item of the reductions: about four items per resident block
+    b->sum_chunk = (int)std::min<int64_t>(
+        lbmp::kBatchMaxChunk,
+        std::max<int64_t>(1, b->total_nodes / ((int64_t)lbmp::kReadBX * 12 * b->nsm)));
+    std::vector<long long> cum_macro(count + 1, 0);
+    for (int i = 0; i < count; ++i)
+      cum_macro[i + 1] = cum_macro[i] + (long long)((nx[i] + lbmp::kReadBX - 1) / lbmp::kReadBX) *
+                                            ((b->h_inst[i].rows + b->sum_chunk - 1) / b->sum_chunk);
     b->items_macro = cum_macro.back();
+    if (b->items_macro > 0x7fffffffLL) BTRY(bfail(LBMP_EINVAL, "batch too large for the reductions"));
     BTRY(balloc(b, (void **)&b->d_inst, sizeof(BatchInst) * count, "batch descriptors"));
     BTRY(balloc(b, (void **)&b->d_cum_step, sizeof(long long) * (count + 1), "work list"));
     BTRY(balloc(b, (void **)&b->d_cum_macro, sizeof(long long) * (count + 1), "work list"));
@@ -1007,9 +1015,9 @@ lbmp_status lbmp_batch_create(const lbmp_params *pin, int32_t count, const int32
       b->items_cap = work_list(b, min_chunk).back();
       BTRY(balloc(b, (void **)&b->d_item_inst, sizeof(int) * (size_t)b->items_cap, "work-item table"));
     }
-    BTRY(balloc(b, (void **)&b->d_partials, sizeof(double) * lbmp::kNQ * (size_t)b->items_macro,
+    BTRY(balloc(b, (void **)&b->d_partials, sizeof(double) * 2 * (size_t)b->items_macro,
                 "batch partials"));
-    BTRY(balloc(b, (void **)&b->d_results, sizeof(double) * lbmp::kNQ * count, "batch results"));
+    BTRY(balloc(b, (void **)&b->d_results, sizeof(double) * 2 * count, "batch results"));
     int max_mb = 0;
     for (int i = 0; i < count; ++i) max_mb = std::max(max_mb, lbmp::medium_blocks(nx[i], ny[i]));
     BTRY(balloc(b, (void **)&b->d_med_partials, sizeof(double) * lbmp::kNQ * max_mb, "medium partials"));
@@ -1285,24 +1293,18 @@ lbmp_status lbmp_batch_permeability(lbmp_batch *b, double *k_g, double *u_mean) 
     if (!all_fields(b)) return bfail(LBMP_ESTATE, "every instance needs its fields");
     const DeviceScope device_scope(b->device);
     BCK(device_scope.err);
-    cudaError_t e;
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, lbmp::batch_macro_kernel<lbmp::StoreF32>, lbmp::kBatchMacroBX, 0);
-    if (e != cudaSuccess) return bcuda(e, "occupancy");
-    const long long grid = std::min<long long>((long long)std::max(per_sm, 1) * b->nsm, b->items_macro);
     if (b->p.storage == LBMP_STORE_FP32)
-      lbmp::batch_macro_kernel<lbmp::StoreF32><<<(unsigned)grid, lbmp::kBatchMacroBX, 0, b->stream>>>(
-          b->d_inst, b->d_cum_macro, b->count, b->parity, b->d_partials);
+      lbmp::batch_sums_kernel<lbmp::StoreF32><<<(unsigned)b->items_macro, lbmp::kReadBX, 0, b->stream>>>(
+          b->h_inst[0].a, b->d_inst, b->d_cum_macro, b->count, b->sum_chunk, b->parity, b->d_partials);
     else
-      lbmp::batch_macro_kernel<lbmp::StoreF16><<<(unsigned)grid, lbmp::kBatchMacroBX, 0, b->stream>>>(
-          b->d_inst, b->d_cum_macro, b->count, b->parity, b->d_partials);
+      lbmp::batch_sums_kernel<lbmp::StoreF16><<<(unsigned)b->items_macro, lbmp::kReadBX, 0, b->stream>>>(
+          b->h_inst[0].a, b->d_inst, b->d_cum_macro, b->count, b->sum_chunk, b->parity, b->d_partials);
     BCK(cudaGetLastError());
-    lbmp::batch_finalize_kernel<<<b->count, 256, 0, b->stream>>>(b->d_cum_macro, b->d_partials,
+    lbmp::batch_finalize_kernel<<<b->count, lbmp::kReadBX, 0, b->stream>>>(b->d_cum_macro, b->d_partials,
                                                                   b->d_results);
     BCK(cudaGetLastError());
     b->launches += 2;
-    std::vector<double> res((size_t)b->count * lbmp::kNQ);
+    std::vector<double> res((size_t)b->count * 2);
     BCK(cudaMemcpyAsync(res.data(), b->d_results, res.size() * sizeof(double),
                         cudaMemcpyDeviceToHost, b->stream));
     BCK(cudaStreamSynchronize(b->stream));
@@ -1310,8 +1312,8 @@ lbmp_status lbmp_batch_permeability(lbmp_batch *b, double *k_g, double *u_mean) 
     const double nu = (p.tau - 0.5) / 3.0 / p.J;
     lbmp_status st = LBMP_OK;
     for (int i = 0; i < b->count; ++i) {
-      const double *r = res.data() + (size_t)i * lbmp::kNQ;
-      if (r[5] != 0.0) st = bfail(LBMP_ENAN, "instance %d has non-finite velocities", i);
+      const double *r = res.data() + (size_t)i * 2;
+      if (r[1] != 0.0) st = bfail(LBMP_ENAN, "instance %d has non-finite velocities", i);
       const double um = r[0] / (double)b->fluid_nodes[i];
       double g = p.Gx;
       if (p.bc_x == LBMP_BCX_PRESSURE)
@@ -1344,9 +1346,7 @@ lbmp_status lbmp_batch_populations(lbmp_batch *b, int32_t i, double *f, int32_t 
       BCK(cudaMalloc(&tmp, n * sizeof(double)));
       dst = (double *)tmp;
     }
-    lbmp::MacroOut o{};
-    o.pops = dst;
-    cudaError_t e = lbmp::launch_macro(b->p.storage, a, I.buf[b->parity], I.med, o, b->stream);
+    cudaError_t e = lbmp::launch_pops(b->p.storage, a, I.buf[b->parity], I.med, dst, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e == cudaSuccess && tmp) e = cudaMemcpy(f, tmp, n * sizeof(double), cudaMemcpyDeviceToHost);
     if (tmp) cudaFree(tmp);

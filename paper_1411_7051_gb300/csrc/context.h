@@ -29,10 +29,12 @@ struct lbmp_ctx {
   double *partials = nullptr;
   int partials_blocks = 0;
   double *results = nullptr;    // device, kNQ doubles
-  double *h_results = nullptr;  // pinned host, kNQ doubles
+  double *h_results = nullptr;  // pinned host, kNQ doubles (read-outs write them in place)
+  unsigned *h_err = nullptr;    // pinned host, behind h_results: copy of *d_err
   unsigned long long *d_hist = nullptr;  // velocity histogram counts (allocated on first use)
   unsigned *d_flag = nullptr;
   unsigned long long *d_tctr = nullptr;  // time level for the stochastic rounding
+  unsigned *d_done = nullptr;            // blocks done in a reduction (0 between launches)
   unsigned *d_err = nullptr;             // raised by a bounded wait that gave up
   int nsm = 1;                           // SMs of the device
   bool staged = true;            // staged kernel (else direct or wide)

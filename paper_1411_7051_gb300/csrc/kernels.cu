@@ -15,6 +15,7 @@
 
 #include "kernels.h"
 #include "lattice.cuh"
+#include "pairs.cuh"
 #include "staged.cuh"
 #include "wide.cuh"
 
@@ -22,7 +23,7 @@ namespace lbmp {
 
 constexpr int kStepBX = 128;   // threads per block along x
 constexpr int kStepNPT = 2;    // nodes per thread, strided by kStepBX
-constexpr int kMacroBX = 256;
+constexpr int kLoadBX = 256;
 constexpr int kMediumBX = 256;
 
 // ------------------------------------------------------------- step kernel
@@ -234,163 +235,6 @@ __device__ __forceinline__ void block_reduce_store(double v[kNQ], double *partia
   }
 }
 
-// ------------------------------------------------ FP32-pair arithmetic
-// Pairs of FP32 numbers (value = hi + lo) carrying ~44 significant bits:
-// exact sums (Knuth's two-sum) and exact products (fma of the product and
-// its negation), the standard error-free transformations.  FP64 arithmetic
-// runs at ~1/64 of the FP32 rate on this GPU; the precompute and the
-// per-thread parts of the reductions use these pairs instead.
-struct F2 {
-  float hi, lo;
-};
-__device__ __forceinline__ F2 two_sum(float a, float b) {
-  const float s = __fadd_rn(a, b);
-  const float bb = __fsub_rn(s, a);
-  const float e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
-  return {s, e};
-}
-__device__ __forceinline__ F2 fast_two_sum(float a, float b) {  // |a| >= |b|
-  const float s = __fadd_rn(a, b);
-  return {s, __fsub_rn(b, __fsub_rn(s, a))};
-}
-__device__ __forceinline__ F2 two_prod(float a, float b) {
-  const float p = __fmul_rn(a, b);
-  return {p, __fmaf_rn(a, b, -p)};
-}
-__device__ __forceinline__ F2 f2_add(F2 x, F2 y) {
-  F2 s = two_sum(x.hi, y.hi);
-  return fast_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(x.lo, y.lo)));
-}
-__device__ __forceinline__ F2 f2_mul(F2 x, F2 y) {
-  F2 p = two_prod(x.hi, y.hi);
-  const float c = __fmaf_rn(x.hi, y.lo, __fmul_rn(x.lo, y.hi));
-  return fast_two_sum(p.hi, __fadd_rn(p.lo, c));
-}
-// n / d from an approximate reciprocal r of d.hi (relative error e ~ 2^-23):
-// q1 = n.hi r is off by ~e, the remainder n - q1 d is formed exactly enough
-// (~2^-48 of n), and its quotient by the same r corrects q1 to a relative
-// error of order e^2 -- one Newton step on the quotient.
-__device__ __forceinline__ F2 f2_div(F2 n, F2 d) {
-  const float r = rcp_approx(d.hi);
-  const float q1 = __fmul_rn(n.hi, r);
-  const F2 qd = f2_mul({q1, 0.0f}, d);           // q1 d
-  const F2 rem = f2_add(n, {-qd.hi, -qd.lo});     // n - q1 d
-  return fast_two_sum(q1, __fmul_rn(rem.hi, r));
-}
-// acc += x (x an FP32 value)
-__device__ __forceinline__ void f2_acc(F2 &acc, float x) {
-  const F2 s = two_sum(acc.hi, x);
-  acc = fast_two_sum(s.hi, __fadd_rn(s.lo, acc.lo));
-}
-
-// ------------------------------------------- macroscopic / reduction kernel
-// Rows blockIdx.y, blockIdx.y + gridDim.y, ...: each thread adds the terms
-// of its nodes (some 27 at 4096^2) one by one in FP32 pairs and takes part
-// in one FP64 block reduction at the end (FP64 arithmetic is slow on this
-// GPU: a reduction tree per node cost six times the per-node work, and FP64
-// per-node sums 0.48 ms at 4096^2).  The squares are exact products, the
-// velocity differences of the residual exact sums; a thread's pair sums
-// are good to ~2^-44 relative.
-// Four resident blocks a SM (64 registers a thread; 2 at the compiler's own
-// 116): 0.37 -> 0.28 ms a lbmp_permeability call at 4096^2.
-template <class S>
-__global__ void __launch_bounds__(kMacroBX, 4)
-    macro_kernel(const StepArgs a, const typename S::T *__restrict__ fin,
-                 const float2 *__restrict__ med, const MacroOut o) {
-  const int x = blockIdx.x * kMacroBX + threadIdx.x;
-  const long long n = (long long)a.nx * a.ny;
-  F2 sux = {0.0f, 0.0f}, suy = {0.0f, 0.0f}, sdr = {0.0f, 0.0f}, su2 = {0.0f, 0.0f},
-     sdu = {0.0f, 0.0f};
-  unsigned nonfinite = 0;
-  for (int y = blockIdx.y; y < a.ny && x < a.nx; y += gridDim.y) {
-    const bool wall = a.walls && (y == 0 || y == a.ny - 1);
-    const long long j = (long long)y * a.nx + x;
-    if (wall) {
-      if (o.rho) o.rho[j] = 0.0;
-      if (o.ux) o.ux[j] = 0.0;
-      if (o.uy) o.uy[j] = 0.0;
-      if (o.pops)
-        for (int i = 0; i < 9; ++i) o.pops[i * n + j] = 0.0;
-      continue;
-    }
-    float d[9];
-    const long long jp = (long long)y * a.pitch + x;
-    const float2 m = med[jp];
-    pull_node<S>(fin, a, x, y, d);
-    const bool col = a.pressure && (x == 0 || x == a.nx - 1);
-    NodeState s;
-    if (a.kn0) {  // dynamic Kn
-      if (col) pressure_node<S, true>(fin, med, a, x, y, m.x, d);
-      s = node_state<true>(d, m.x, m.y, a, a.kn0[jp]);
-    } else {
-      if (col) pressure_node<S, false>(fin, med, a, x, y, m.x, d);
-      s = node_state<false>(d, m.x, m.y, a);
-    }
-    const float drho = s.drho_s * a.inv_scale;
-    if (o.rho) o.rho[j] = (double)s.rho;
-    if (o.ux) o.ux[j] = (double)s.ux;
-    if (o.uy) o.uy[j] = (double)s.uy;
-    if (o.pops) {
-      const double r0 = (double)a.rho0;
-      const double w[9] = {4.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0,  1.0 / 9.0, 1.0 / 9.0,
-                           1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0, 1.0 / 36.0};
-      const double is = (double)a.inv_scale;
-      for (int i = 0; i < 9; ++i) o.pops[i * n + j] = w[i] * r0 + (double)d[i] * is;
-    }
-    if (o.partials) {
-      const bool finite = isfinite(s.ux) && isfinite(s.uy) && isfinite(s.rho);
-      if (finite) {
-        f2_acc(sux, s.ux);
-        f2_acc(suy, s.uy);
-        f2_acc(sdr, drho);
-        su2 = f2_add(su2, f2_add(two_prod(s.ux, s.ux), two_prod(s.uy, s.uy)));
-      } else {
-        ++nonfinite;
-      }
-      if (o.uprev) {
-        const float2 up = o.uprev[jp];
-        if (finite) {
-          const F2 dx = two_sum(s.ux, -up.x), dy = two_sum(s.uy, -up.y);
-          sdu = f2_add(sdu, f2_add(f2_mul(dx, dx), f2_mul(dy, dy)));
-        }
-        if (o.update_prev) o.uprev[jp] = make_float2(s.ux, s.uy);
-      }
-    }
-  }
-  if (o.partials) {
-    double v[kNQ] = {(double)sux.hi + (double)sux.lo, (double)suy.hi + (double)suy.lo,
-                     (double)sdr.hi + (double)sdr.lo, (double)su2.hi + (double)su2.lo,
-                     (double)sdu.hi + (double)sdu.lo, (double)nonfinite};
-    block_reduce_store<kMacroBX>(v, o.partials);
-  }
-}
-
-// Up to 16 blocks of 256 threads on each of 152 SMs.
-constexpr int kMacroMaxBlocks = 16 * 152;
-
-static dim3 macro_grid(const StepArgs &a) {
-  const int gx = (a.nx + kMacroBX - 1) / kMacroBX;
-  const int gy = std::max(1, std::min(a.ny, kMacroMaxBlocks / gx));
-  return dim3(gx, gy);
-}
-
-int macro_blocks(const StepArgs &a) {
-  const dim3 g = macro_grid(a);
-  return (int)(g.x * g.y);
-}
-
-int hist_blocks(const StepArgs &a) { return ((a.nx + kMacroBX - 1) / kMacroBX) * a.ny; }
-
-cudaError_t launch_macro(int storage, const StepArgs &a, const void *fin,
-                         const float2 *med, const MacroOut &o, cudaStream_t s) {
-  const dim3 block(kMacroBX), grid = macro_grid(a);
-  if (storage == 0)
-    macro_kernel<StoreF32><<<grid, block, 0, s>>>(a, (const float *)fin, med, o);
-  else
-    macro_kernel<StoreF16><<<grid, block, 0, s>>>(a, (const __half *)fin, med, o);
-  return cudaGetLastError();
-}
-
 // ------------------------------------------------------------- finalize
 constexpr int kFinBX = 256;
 
@@ -421,106 +265,6 @@ __global__ void __launch_bounds__(kFinBX)
 cudaError_t launch_finalize(const double *partials, int nblocks, int nq, double *out,
                             cudaStream_t s, unsigned max_mask) {
   finalize_kernel<<<1, kFinBX, 0, s>>>(partials, nblocks, nq, out, max_mask);
-  return cudaGetLastError();
-}
-
-// ------------------------------------------- normalised-velocity histogram
-// |u| of node (x, y) in FP64 from the FP32 velocity of node_state (as the
-// macroscopic kernel reports it), every operation rounded separately so
-// that the bin decisions can be replayed exactly on the host.
-template <class S, bool DYN>
-__device__ __forceinline__ double node_speed(const typename S::T *__restrict__ fin,
-                                             const float2 *__restrict__ med, const StepArgs &a,
-                                             int x, int y) {
-  float d[9];
-  const long long jp = (long long)y * a.pitch + x;
-  const float2 m = med[jp];
-  pull_node<S>(fin, a, x, y, d);
-  if (a.pressure && (x == 0 || x == a.nx - 1)) pressure_node<S, DYN>(fin, med, a, x, y, m.x, d);
-  const NodeState s = node_state<DYN>(d, m.x, m.y, a, DYN ? a.kn0[jp] : 0.0f);
-  const double ux = s.ux, uy = s.uy;
-  return __dsqrt_rn(__dadd_rn(__dmul_rn(ux, ux), __dmul_rn(uy, uy)));
-}
-
-// Pass 1: block maxima of |u| over the fluid rows into partials[block].
-template <class S, bool DYN>
-__global__ void __launch_bounds__(kMacroBX)
-    speed_max_kernel(const StepArgs a, const typename S::T *__restrict__ fin,
-                     const float2 *__restrict__ med, double *__restrict__ partials) {
-  const int y = blockIdx.y;
-  const int x = blockIdx.x * kMacroBX + threadIdx.x;
-  double v = 0.0;
-  if (x < a.nx && !(a.walls && (y == 0 || y == a.ny - 1))) v = node_speed<S, DYN>(fin, med, a, x, y);
-  if (!(v >= 0.0)) v = INFINITY;  // a non-finite speed poisons the maximum
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v = fmax(v, __shfl_down_sync(0xffffffffu, v, off));
-  __shared__ double red[kMacroBX / 32];
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kMacroBX / 32; ++w) t = fmax(t, red[w]);
-    partials[(long long)blockIdx.y * gridDim.x + blockIdx.x] = t;
-  }
-}
-
-// Pass 2: bin k = min(floor(|u| / umax * nbins), nbins - 1) (0 if umax is
-// 0), counted per block in shared memory, then added to counts.
-template <class S, bool DYN>
-__global__ void __launch_bounds__(kMacroBX)
-    histogram_kernel(const StepArgs a, const typename S::T *__restrict__ fin,
-                     const float2 *__restrict__ med, double umax, int nbins,
-                     unsigned long long *__restrict__ counts) {
-  __shared__ unsigned sh[kMaxHistBins];
-  for (int k = threadIdx.x; k < nbins; k += kMacroBX) sh[k] = 0u;
-  __syncthreads();
-  const int y = blockIdx.y;
-  const int x = blockIdx.x * kMacroBX + threadIdx.x;
-  if (x < a.nx && !(a.walls && (y == 0 || y == a.ny - 1))) {
-    int k = 0;
-    if (umax > 0.0) {
-      const double u0 = __ddiv_rn(node_speed<S, DYN>(fin, med, a, x, y), umax);
-      const double f = floor(__dmul_rn(u0, (double)nbins));
-      k = f >= (double)(nbins - 1) ? nbins - 1 : (int)f;
-    }
-    atomicAdd(&sh[k], 1u);
-  }
-  __syncthreads();
-  for (int k = threadIdx.x; k < nbins; k += kMacroBX)
-    if (sh[k]) atomicAdd(counts + k, (unsigned long long)sh[k]);
-}
-
-cudaError_t launch_speed_max(int storage, const StepArgs &a, const void *fin, const float2 *med,
-                             double *partials, cudaStream_t s) {
-  dim3 block(kMacroBX);
-  dim3 grid((a.nx + kMacroBX - 1) / kMacroBX, a.ny);
-  const bool dyn = a.kn0 != nullptr;
-  if (storage == 0) {
-    if (dyn) speed_max_kernel<StoreF32, true><<<grid, block, 0, s>>>(a, (const float *)fin, med, partials);
-    else speed_max_kernel<StoreF32, false><<<grid, block, 0, s>>>(a, (const float *)fin, med, partials);
-  } else {
-    if (dyn) speed_max_kernel<StoreF16, true><<<grid, block, 0, s>>>(a, (const __half *)fin, med, partials);
-    else speed_max_kernel<StoreF16, false><<<grid, block, 0, s>>>(a, (const __half *)fin, med, partials);
-  }
-  return cudaGetLastError();
-}
-
-cudaError_t launch_histogram(int storage, const StepArgs &a, const void *fin, const float2 *med,
-                             double umax, int nbins, unsigned long long *counts, cudaStream_t s) {
-  dim3 block(kMacroBX);
-  dim3 grid((a.nx + kMacroBX - 1) / kMacroBX, a.ny);
-  const bool dyn = a.kn0 != nullptr;
-  if (storage == 0) {
-    if (dyn)
-      histogram_kernel<StoreF32, true><<<grid, block, 0, s>>>(a, (const float *)fin, med, umax, nbins, counts);
-    else
-      histogram_kernel<StoreF32, false><<<grid, block, 0, s>>>(a, (const float *)fin, med, umax, nbins, counts);
-  } else {
-    if (dyn)
-      histogram_kernel<StoreF16, true><<<grid, block, 0, s>>>(a, (const __half *)fin, med, umax, nbins, counts);
-    else
-      histogram_kernel<StoreF16, false><<<grid, block, 0, s>>>(a, (const __half *)fin, med, umax, nbins, counts);
-  }
   return cudaGetLastError();
 }
 
@@ -724,42 +468,15 @@ cudaError_t launch_medium(const double *eps, const double *k_i, const double *kn
   return cudaGetLastError();
 }
 
-// ------------------------------------------------- apparent permeability
-// k_a of every node of the fluid rows as the step sees it: 1 / (stored
-// 1/k_a), or with a dynamic Kn 1 / ((1/k_i) / f_c(Kn0)) at the pressure
-// p0 (q = 1) with the step's own FP32 f_c.  Plate rows read 0.
-__global__ void __launch_bounds__(kMediumBX)
-    ka_kernel(const float2 *__restrict__ med, const float *__restrict__ kn0, int nx, int ny,
-              int pitch, int y_lo, int y_hi, int kn_model, double *__restrict__ ka) {
-  const int y = blockIdx.y;
-  const int x = blockIdx.x * kMediumBX + threadIdx.x;
-  if (x >= nx) return;
-  double v = 0.0;
-  if (y >= y_lo && y < y_hi) {
-    const long long jp = (long long)y * pitch + x;
-    float inv = med[jp].y;
-    if (kn0) inv = inv_ka_dynamic(inv, kn0[jp], kn_model);  // the step's form at p = p0
-    v = 1.0 / (double)inv;  // inf for an open pore (1/k_a = 0)
-  }
-  ka[(long long)y * nx + x] = v;
-}
-
-cudaError_t launch_ka(const float2 *med, const float *kn0, int nx, int ny, int pitch, int y_lo,
-                      int y_hi, int kn_model, double *ka, cudaStream_t s) {
-  dim3 grid((nx + kMediumBX - 1) / kMediumBX, ny);
-  ka_kernel<<<grid, kMediumBX, 0, s>>>(med, kn0, nx, ny, pitch, y_lo, y_hi, kn_model, ka);
-  return cudaGetLastError();
-}
-
 // ----------------------------------------------------- population loading
 // B_j(z) = f_j(z + e_j) when z + e_j is a fluid node (wrapped), f_opp(j)(z)
 // when it lies in a plate row, and 0 (unused) beyond a pressure column.
 template <class S>
-__global__ void __launch_bounds__(kMacroBX)
+__global__ void __launch_bounds__(kLoadBX)
     load_pops_kernel(const StepArgs a, const double *__restrict__ f,
                      typename S::T *__restrict__ buf) {
   const int y = a.y0 + blockIdx.y;
-  const int x = blockIdx.x * kMacroBX + threadIdx.x;
+  const int x = blockIdx.x * kLoadBX + threadIdx.x;
   if (x >= a.nx) return;
   const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -793,8 +510,8 @@ __global__ void __launch_bounds__(kMacroBX)
 
 cudaError_t launch_load_pops(int storage, const StepArgs &a, int rows, const double *f,
                              void *buf, cudaStream_t s) {
-  dim3 block(kMacroBX);
-  dim3 grid((a.nx + kMacroBX - 1) / kMacroBX, rows);
+  dim3 block(kLoadBX);
+  dim3 grid((a.nx + kLoadBX - 1) / kLoadBX, rows);
   if (storage == 0)
     load_pops_kernel<StoreF32><<<grid, block, 0, s>>>(a, f, (float *)buf);
   else

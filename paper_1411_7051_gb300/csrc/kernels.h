@@ -13,16 +13,6 @@ namespace lbmp {
 // count of non-finite nodes.
 constexpr int kNQ = 6;
 
-struct MacroOut {
-  double *rho;       // [ny][nx] or NULL
-  double *ux;        // [ny][nx] or NULL
-  double *uy;        // [ny][nx] or NULL
-  double *pops;      // [9][ny][nx] or NULL
-  float2 *uprev;     // [ny][pitch] velocity snapshot, or NULL
-  int update_prev;   // overwrite uprev with u after reading it
-  double *partials;  // [blocks][kNQ] or NULL (no reduction)
-};
-
 // Beskok-Karniadakis-Civan factor (Eq. 6-7, b = -1); f_c(0) = 1.
 __host__ __device__ inline double fc_bkc(double kn) {
   if (kn == 0.0) return 1.0;
@@ -92,13 +82,25 @@ lbmp_status validate_params(::lbmp_params *p);
 // *tctr += n (one thread).
 cudaError_t launch_bump(unsigned long long *tctr, int n, cudaStream_t s);
 
-// Blocks a macroscopic/reduction launch over all ny rows uses.
+// Read-outs of the level that pulling fin gives, over all rows (a.y0 is
+// ignored; plate rows read 0 and count nowhere).  `done` is a device counter
+// that is 0 between launches, `partials` holds 3 macro_blocks(a) doubles, `out` is
+// pinned host memory (valid after the launch has completed).
 int macro_blocks(const StepArgs &a);
-// Blocks (partials) of the histogram's first pass (one block per 256 nodes
-// of a row).
-int hist_blocks(const StepArgs &a);
-cudaError_t launch_macro(int storage, const StepArgs &a, const void *fin,
-                         const float2 *med, const MacroOut &o, cudaStream_t s);
+// Density and velocity, [ny][nx] float64 each; any output may be NULL.
+cudaError_t launch_fields(int storage, const StepArgs &a, const void *fin, const float2 *med,
+                          double *rho, double *ux, double *uy, cudaStream_t s);
+// Post-stream populations, [9][ny][nx] float64.
+cudaError_t launch_pops(int storage, const StepArgs &a, const void *fin, const float2 *med,
+                        double *pops, cudaStream_t s);
+// out[0] sum u_x, out[2] sum (rho - rho0), out[5] non-finite nodes.
+cudaError_t launch_sums(int storage, const StepArgs &a, const void *fin, const float2 *med,
+                        double *partials, unsigned *done, double *out, cudaStream_t s);
+// out[3] sum |u|^2, out[4] sum |u - u_prev|^2, out[5] non-finite nodes; then
+// u_prev = u ([ny][pitch] float2).
+cudaError_t launch_residual_sums(int storage, const StepArgs &a, const void *fin,
+                                 const float2 *med, float2 *uprev, double *partials,
+                                 unsigned *done, double *out, cudaStream_t s);
 
 // Reduce [nblocks][nq] partials in a fixed order into out[0..nq): by sum,
 // or by max for the quantities whose bit is set in max_mask.
@@ -122,15 +124,17 @@ cudaError_t launch_medium(const double *eps, const double *k_i, const double *kn
 cudaError_t launch_ka(const float2 *med, const float *kn0, int nx, int ny, int pitch, int y_lo,
                       int y_hi, int kn_model, double *ka, cudaStream_t s);
 
-// Normalised-velocity histogram: pass 1 writes the maximum of |u| over the
-// fluid rows of each block (hist_blocks(a) doubles, a.y0 ignored);
-// pass 2 adds the counts of bins min(floor(|u| / umax * nbins), nbins - 1)
+// Normalised-velocity histogram: pass 1 writes max |u| over the fluid rows
+// (infinite if a velocity is not finite) to *umax (device) and out[0] (pinned
+// host); pass 2 adds the counts of bins min(floor(|u| / *umax * nbins), nbins - 1)
 // to counts[0..nbins).  nbins <= kMaxHistBins.
 constexpr int kMaxHistBins = 64;
 cudaError_t launch_speed_max(int storage, const StepArgs &a, const void *fin, const float2 *med,
-                             double *partials, cudaStream_t s);
+                             double *partials, unsigned *done, double *umax, double *out,
+                             cudaStream_t s);
 cudaError_t launch_histogram(int storage, const StepArgs &a, const void *fin, const float2 *med,
-                             double umax, int nbins, unsigned long long *counts, cudaStream_t s);
+                             const double *umax, int nbins, unsigned long long *counts,
+                             cudaStream_t s);
 
 // Inverse of the pull: write a post-collision buffer whose pull gives the
 // post-stream populations f ([9][ny][nx] float64).

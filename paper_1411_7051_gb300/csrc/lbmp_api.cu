@@ -114,6 +114,7 @@ void release(lbmp_ctx *c) {
   cudaFree(c->d_flag);
   cudaFree(c->d_tctr);
   cudaFree(c->d_err);
+  cudaFree(c->d_done);
   cudaFree(c->d_hist);
   if (c->h_results) cudaFreeHost(c->h_results);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -133,37 +134,30 @@ struct DevTemp {
   }
 };
 
-// The flag of the bounded waits (synchronous read).
+// Wait for the stream and read the flag of the bounded waits.
 lbmp_status check_err(lbmp_ctx *c) {
-  unsigned e = 0;
-  LBMP_CK(cudaMemcpyAsync(&e, c->d_err, sizeof(e), cudaMemcpyDeviceToHost, c->stream));
+  LBMP_CK(cudaMemcpyAsync(c->h_err, c->d_err, sizeof(unsigned), cudaMemcpyDeviceToHost, c->stream));
   LBMP_CK(cudaStreamSynchronize(c->stream));
-  if (e) return fail(LBMP_ETIMEOUT, "a bounded wait of the staged step kernel gave up");
+  if (*c->h_err) return fail(LBMP_ETIMEOUT, "a bounded wait of the staged step kernel gave up");
   return LBMP_OK;
 }
 
-// Run the macroscopic/reduction kernel and, when partials are requested,
-// reduce them into c->h_results (synchronous).
-lbmp_status run_macro(lbmp_ctx *c, lbmp::MacroOut o, bool reduce) {
-  StepArgs a = c->args();
-  a.y0 = 0;
-  if (reduce) o.partials = c->partials;
-  LBMP_CK(lbmp::launch_macro(c->p.storage, a, c->buf[c->cur], c->med, o, c->stream));
+// Wait for a read-out (and its sums in c->h_results).
+lbmp_status finish_sums(lbmp_ctx *c) {
   c->launches++;
-  if (reduce) {
-    LBMP_CK(lbmp::launch_finalize(c->partials, lbmp::macro_blocks(a), lbmp::kNQ,
-                                  c->results, c->stream));
-    c->launches++;
-    LBMP_CK(cudaMemcpyAsync(c->h_results, c->results, sizeof(double) * lbmp::kNQ,
-                            cudaMemcpyDeviceToHost, c->stream));
-  }
-  LBMP_CK(cudaStreamSynchronize(c->stream));
   lbmp_status st = check_err(c);
   if (st) return st;
-  if (reduce && c->h_results[5] != 0.0)
+  if (c->h_results[5] != 0.0)
     return fail(LBMP_ENAN, "%.0f fluid nodes have a non-finite density or velocity",
                 c->h_results[5]);
   return LBMP_OK;
+}
+
+// The sums behind k_g and the mass into c->h_results (synchronous).
+lbmp_status run_sums(lbmp_ctx *c) {
+  LBMP_CK(lbmp::launch_sums(c->p.storage, c->args(), c->buf[c->cur], c->med, c->partials,
+                            c->d_done, c->h_results, c->stream));
+  return finish_sums(c);
 }
 
 // One step kernel launch (the variant the context selected).  Steps that
@@ -401,10 +395,7 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     }
     e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaStreamCreate (capture)"));
-    StepArgs a = c->args();
-    a.y0 = 0;
-    c->partials_blocks = std::max({lbmp::macro_blocks(a), lbmp::hist_blocks(a),
-                                   lbmp::medium_blocks(p.nx, p.ny)});
+    c->partials_blocks = std::max(lbmp::macro_blocks(c->args()), lbmp::medium_blocks(p.nx, p.ny));
     LBMP_TRY(dalloc(c, &c->buf[0], c->buf_bytes(), "population buffer A"));
     LBMP_TRY(dalloc(c, &c->buf[1], c->buf_bytes(), "population buffer B"));
     LBMP_TRY(dalloc(c, (void **)&c->med, (size_t)c->plane * sizeof(float2), "medium"));
@@ -419,8 +410,12 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     LBMP_TRY(dalloc(c, (void **)&c->d_err, sizeof(unsigned), "wait error flag"));
     e = cudaMemset(c->d_err, 0, sizeof(unsigned));
     if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMemset"));
-    e = cudaMallocHost((void **)&c->h_results, lbmp::kNQ * sizeof(double));
+    LBMP_TRY(dalloc(c, (void **)&c->d_done, sizeof(unsigned), "block counter"));
+    e = cudaMemset(c->d_done, 0, sizeof(unsigned));
+    if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMemset"));
+    e = cudaMallocHost((void **)&c->h_results, (lbmp::kNQ + 1) * sizeof(double));
     if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMallocHost"));
+    c->h_err = reinterpret_cast<unsigned *>(c->h_results + lbmp::kNQ);
 #undef LBMP_TRY
     *out = c;
     return LBMP_OK;
@@ -614,21 +609,20 @@ lbmp_status lbmp_macroscopic(lbmp_ctx *c, double *rho, double *ux, double *uy,
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
     const size_t n = (size_t)c->p.nx * c->p.ny;
-    lbmp::MacroOut o{};
+    double *o_rho = rho, *o_ux = ux, *o_uy = uy;
     DevTemp tmp;
     if (where == LBMP_HOST) {
       cudaError_t e = cudaMalloc(&tmp.ptr, 3 * n * sizeof(double));
       if (e != cudaSuccess) return cuda_fail(e, "staging buffer");
       double *t = (double *)tmp.ptr;
-      o.rho = rho ? t : nullptr;
-      o.ux = ux ? t + n : nullptr;
-      o.uy = uy ? t + 2 * n : nullptr;
-    } else {
-      o.rho = rho;
-      o.ux = ux;
-      o.uy = uy;
+      o_rho = rho ? t : nullptr;
+      o_ux = ux ? t + n : nullptr;
+      o_uy = uy ? t + 2 * n : nullptr;
     }
-    st = run_macro(c, o, false);
+    LBMP_CK(lbmp::launch_fields(c->p.storage, c->args(), c->buf[c->cur], c->med, o_rho, o_ux,
+                                o_uy, c->stream));
+    c->launches++;
+    st = check_err(c);
     if (st) return st;
     if (where == LBMP_HOST) {
       double *t = (double *)tmp.ptr;
@@ -681,16 +675,16 @@ lbmp_status lbmp_populations(lbmp_ctx *c, double *f, int32_t where) {
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
     const size_t n = (size_t)c->p.nx * c->p.ny * 9;
-    lbmp::MacroOut o{};
+    double *pops = f;
     DevTemp tmp;
     if (where == LBMP_HOST) {
       cudaError_t e = cudaMalloc(&tmp.ptr, n * sizeof(double));
       if (e != cudaSuccess) return cuda_fail(e, "staging buffer");
-      o.pops = (double *)tmp.ptr;
-    } else {
-      o.pops = f;
+      pops = (double *)tmp.ptr;
     }
-    st = run_macro(c, o, false);
+    LBMP_CK(lbmp::launch_pops(c->p.storage, c->args(), c->buf[c->cur], c->med, pops, c->stream));
+    c->launches++;
+    st = check_err(c);
     if (st) return st;
     if (where == LBMP_HOST)
       LBMP_CK(cudaMemcpy(f, tmp.ptr, n * sizeof(double), cudaMemcpyDeviceToHost));
@@ -736,8 +730,7 @@ lbmp_status lbmp_permeability(lbmp_ctx *c, double *k_g, double *u_mean) {
     const DeviceScope device_scope(c->device);
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
-    lbmp::MacroOut o{};
-    st = run_macro(c, o, true);
+    st = run_sums(c);
     if (st) return st;
     const lbmp_params &p = c->p;
     const double um = c->h_results[0] / (double)c->fluid_nodes;
@@ -769,28 +762,21 @@ lbmp_status lbmp_velocity_histogram(lbmp_ctx *c, int32_t nbins, double *umax,
                   "histogram counts");
       if (st) return st;
     }
-    StepArgs a = c->args();
-    a.y0 = 0;
-    LBMP_CK(lbmp::launch_speed_max(c->p.storage, a, c->buf[c->cur], c->med, c->partials,
-                                   c->stream));
-    LBMP_CK(lbmp::launch_finalize(c->partials, lbmp::hist_blocks(a), 1, c->results, c->stream,
-                                  1u));
-    LBMP_CK(cudaMemcpyAsync(c->h_results, c->results, sizeof(double), cudaMemcpyDeviceToHost,
-                            c->stream));
-    LBMP_CK(cudaStreamSynchronize(c->stream));
-    const double um = c->h_results[0];
-    if (!std::isfinite(um)) return fail(LBMP_ENAN, "a fluid node has a non-finite velocity");
+    const StepArgs a = c->args();
     LBMP_CK(cudaMemsetAsync(c->d_hist, 0, lbmp::kMaxHistBins * sizeof(unsigned long long),
                             c->stream));
-    LBMP_CK(lbmp::launch_histogram(c->p.storage, a, c->buf[c->cur], c->med, um, nbins, c->d_hist,
-                                   c->stream));
-    c->launches += 3;
+    LBMP_CK(lbmp::launch_speed_max(c->p.storage, a, c->buf[c->cur], c->med, c->partials, c->d_done,
+                                   c->results, c->h_results, c->stream));
+    LBMP_CK(lbmp::launch_histogram(c->p.storage, a, c->buf[c->cur], c->med, c->results, nbins,
+                                   c->d_hist, c->stream));
+    c->launches += 2;
     unsigned long long h[lbmp::kMaxHistBins];
     LBMP_CK(cudaMemcpyAsync(h, c->d_hist, (size_t)nbins * sizeof(unsigned long long),
                             cudaMemcpyDeviceToHost, c->stream));
-    LBMP_CK(cudaStreamSynchronize(c->stream));
     st = check_err(c);
     if (st) return st;
+    const double um = c->h_results[0];
+    if (!std::isfinite(um)) return fail(LBMP_ENAN, "a fluid node has a non-finite velocity");
     for (int k = 0; k < nbins; ++k) counts[k] = (int64_t)h[k];
     if (umax) *umax = um;
     return LBMP_OK;
@@ -807,10 +793,9 @@ lbmp_status lbmp_residual(lbmp_ctx *c, double *r) {
     const DeviceScope device_scope(c->device);
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
-    lbmp::MacroOut o{};
-    o.uprev = c->uprev;
-    o.update_prev = 1;
-    st = run_macro(c, o, true);
+    LBMP_CK(lbmp::launch_residual_sums(c->p.storage, c->args(), c->buf[c->cur], c->med, c->uprev,
+                                       c->partials, c->d_done, c->h_results, c->stream));
+    st = finish_sums(c);
     if (st) return st;
     *r = std::sqrt(c->h_results[4]) / std::sqrt(c->h_results[3]);
     return LBMP_OK;
@@ -827,8 +812,7 @@ lbmp_status lbmp_mass(lbmp_ctx *c, double *m) {
     const DeviceScope device_scope(c->device);
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
-    lbmp::MacroOut o{};
-    st = run_macro(c, o, true);
+    st = run_sums(c);
     if (st) return st;
     *m = (double)c->fluid_nodes * c->p.rho0 + c->h_results[2];
     return LBMP_OK;
