@@ -19,8 +19,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_lib")
 LIB = os.path.join(OUT_DIR, "liblbmp.so")
-SOURCES = ["kernels.cu", "fused.cu", "readout.cu", "lbmp_api.cu", "noalloc.cu", "batch.cu", "adjoint.cu"]
-HEADERS = ["lattice.cuh", "kernels.h", "pairs.cuh", "readout.cuh", "staged.cuh", "fused.cuh", "wide.cuh", "context.h", "nvtx_range.h", "device_scope.h"]
+SOURCES = ["kernels.cu", "fused.cu", "tile.cu", "readout.cu", "lbmp_api.cu", "noalloc.cu", "batch.cu", "adjoint.cu"]
+HEADERS = ["chain.cuh", "lattice.cuh", "kernels.h", "pairs.cuh", "readout.cuh", "staged.cuh", "fused.cuh", "tile.cuh", "wide.cuh", "context.h", "nvtx_range.h", "device_scope.h"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 NVCC_FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC,-O2",
               "-Xptxas", "-O3", "--expt-relaxed-constexpr"]
@@ -44,7 +44,7 @@ def source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-STEP_KERNEL_FILES = ["kernels.cu", "fused.cu", "fused.cuh", "kernels.h", "lattice.cuh", "staged.cuh"]
+STEP_KERNEL_FILES = ["kernels.cu", "chain.cuh", "fused.cu", "fused.cuh", "kernels.h", "lattice.cuh", "staged.cuh"]
 ADJOINT_KERNEL_FILES = ["adjoint.cu", "kernels.h", "lattice.cuh"]
 BATCH_KERNEL_FILES = ["batch.cu", "fused.cuh", "kernels.h", "lattice.cuh", "staged.cuh"]
 

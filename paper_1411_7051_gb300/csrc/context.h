@@ -40,6 +40,10 @@ struct lbmp_ctx {
   bool staged = true;            // staged kernel (else direct or wide)
   bool wide = false;             // wide FP16 kernel
   bool fused = false;            // lbmp_step pairs its steps (two per launch)
+  bool tiled = false;            // ... or runs tile.levels of them per launch
+  lbmp::TilePlan tile{};
+  // steps of a full launch of lbmp_step
+  int per_launch() const { return tiled ? tile.levels : (fused ? 2 : 1); }
   bool sr = false;
   bool fields_set = false;
   int64_t steps = 0;
@@ -52,7 +56,7 @@ struct lbmp_ctx {
   int fault_alloc_at = 0;       // simulated allocation failure (testing)
   int drop_tile = -1;           // withheld tile of the staged kernel (testing)
   // step graphs: [l][cur] replays 2^l launches starting from buffer cur (of
-  // two steps each with `fused`); odd[cur] the single step left over then
+  // per_launch() steps each); odd[cur] the single step left over with `fused`
   cudaGraphExec_t graph[6][2] = {};
   cudaGraphExec_t odd[2] = {};
 

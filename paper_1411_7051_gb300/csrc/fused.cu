@@ -52,11 +52,11 @@ static cudaError_t launch_fused_q(const StepArgs &a, int rows, const void *fin, 
       cudaFuncSetAttribute(fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>,
                            cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   if (attr != cudaSuccess) return attr;
-  fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>
-      <<<(plan.tasks + kFusedWarps - 1) / kFusedWarps, kFusedWarps * 32, C::kSmemBytes, s>>>(
+  return launch_chained(fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>,
+                        dim3((plan.tasks + kFusedWarps - 1) / kFusedWarps), dim3(kFusedWarps * 32),
+                        C::kSmemBytes, s,
           a, (const typename S::T *)fin, (typename S::T *)fout, med, tctr, k, rows, plan.seg,
           plan.f, plan.edges, plan.tasks, mom1, mom2);
-  return cudaGetLastError();
 }
 
 template <class S, bool SR, bool DYN, bool MOM>

@@ -33,6 +33,7 @@
 
 #include <cmath>
 
+#include "chain.cuh"
 #include "lattice.cuh"
 #include "staged.cuh"
 
@@ -116,7 +117,7 @@ template <>
 struct LaneRaw<StoreF32, float2> {
   using R = float2;
   static __device__ __forceinline__ R load(const float *p) {
-    return __ldg(reinterpret_cast<const float2 *>(p));
+    return *reinterpret_cast<const float2 *>(p);
   }
   static __device__ __forceinline__ R from_left(R v) {  // sources at x - 1
     return make_float2(__shfl_up_sync(0xffffffffu, v.y, 1), v.x);
@@ -133,7 +134,7 @@ struct LaneRaw<StoreF32, float2> {
 template <>
 struct LaneRaw<StoreF32, float> {
   using R = float;
-  static __device__ __forceinline__ R load(const float *p) { return __ldg(p); }
+  static __device__ __forceinline__ R load(const float *p) { return *p; }
   static __device__ __forceinline__ R from_left(R v) { return __shfl_up_sync(0xffffffffu, v, 1); }
   static __device__ __forceinline__ R from_right(R v) {
     return __shfl_down_sync(0xffffffffu, v, 1);
@@ -142,13 +143,14 @@ struct LaneRaw<StoreF32, float> {
   template <bool SR>
   static __device__ __forceinline__ R round(float v, uint32_t, int) { return v; }
   static __device__ __forceinline__ void store(float *p, R v) { put_global(p, v); }
+  static __device__ __forceinline__ void keep(float *p, R v) { *p = v; }  // any memory
 };
 
 template <>
 struct LaneRaw<StoreF16, float2> {
   using R = uint32_t;  // half of node x in the low 16 bits, of node x + 1 in the high ones
   static __device__ __forceinline__ R load(const __half *p) {
-    return __ldg(reinterpret_cast<const uint32_t *>(p));
+    return *reinterpret_cast<const uint32_t *>(p);
   }
   static __device__ __forceinline__ R from_left(R v) {
     return __byte_perm(__shfl_up_sync(0xffffffffu, v, 1), v, 0x5432);
@@ -180,7 +182,7 @@ template <>
 struct LaneRaw<StoreF16, float> {
   using R = uint32_t;  // in the low 16 bits
   static __device__ __forceinline__ R load(const __half *p) {
-    return __ldg(reinterpret_cast<const unsigned short *>(p));
+    return *reinterpret_cast<const unsigned short *>(p);
   }
   static __device__ __forceinline__ R from_left(R v) { return __shfl_up_sync(0xffffffffu, v, 1); }
   static __device__ __forceinline__ R from_right(R v) {
@@ -202,6 +204,9 @@ struct LaneRaw<StoreF16, float> {
   }
   static __device__ __forceinline__ void store(__half *p, R v) {
     put_global(p, (unsigned short)v);
+  }
+  static __device__ __forceinline__ void keep(__half *p, R v) {
+    *reinterpret_cast<unsigned short *>(p) = (unsigned short)v;
   }
 };
 
@@ -314,7 +319,7 @@ __device__ __forceinline__ void lane_collide(V d[9], const NodeStateT<V> &s, con
 // below x_lo or from x_hi on are stored.  MOM: the moments of levels t and t + 1
 // go to mom1 and mom2.
 template <class S, bool SR, bool DYN, bool MOM, class V>
-__device__ __forceinline__ void fused_edges(const StepArgs &a, const typename S::T *__restrict__ fin,
+__device__ __forceinline__ void fused_edges(const StepArgs &a, const typename S::T *fin,
                                             typename S::T *__restrict__ fout,
                                             const float2 *__restrict__ med, int win, int x_lo,
                                             int x_hi, int s0, int s1, int seg, int y_end,
@@ -566,7 +571,7 @@ __device__ __forceinline__ void level_row(typename LaneRaw<S, float2>::R t[9][Q]
 // The walk of an interior strip (first column c0) over rows [s0, s1), as
 // fused_walk, with the rows of level t copied ahead.
 template <class S, bool SR, bool DYN, bool MOM, int Q>
-__device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S::T *__restrict__ fin,
+__device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S::T *fin,
                                             typename S::T *__restrict__ fout,
                                             const float2 *__restrict__ med, int c0, int s0, int s1,
                                             int y_end, uint32_t ts1, uint32_t ts2,
@@ -772,7 +777,7 @@ inline double fused_cost(int seg, double w) {
 // One warp's task: strip `strip` of the segment that starts at row s0, seg
 // rows high at most; strip < 0: the edges of that segment and the next per - 1.
 template <class S, bool SR, bool DYN, bool MOM, int Q>
-__device__ __forceinline__ void fused_task(const StepArgs &a, const typename S::T *__restrict__ fin,
+__device__ __forceinline__ void fused_task(const StepArgs &a, const typename S::T *fin,
                                            typename S::T *__restrict__ fout,
                                            const float2 *__restrict__ med, const FusedStrips &f,
                                            int strip, int s0, int seg, int y_end, uint32_t ts1,
@@ -810,9 +815,9 @@ __device__ __forceinline__ uint32_t level_hash(const StepArgs &a, unsigned long 
 // shorter).  FORCH = a0.forch, as a constant: no branch inside a row.
 template <class S, bool SR, bool DYN, bool MOM, bool FORCH, int Q>
 __global__ void __launch_bounds__(kFusedWarps * 32, FusedCfg<S, Q, DYN>::kBlocks)
-    fused_step_kernel(const StepArgs a0, const typename S::T *__restrict__ fin,
+    fused_step_kernel(const StepArgs a0, const typename S::T *fin,
                       typename S::T *__restrict__ fout, const float2 *__restrict__ med,
-                      const unsigned long long *__restrict__ tctr, int k, int rows, int seg,
+                      const unsigned long long *tctr, int k, int rows, int seg,
                       const FusedStrips f, int edges, int tasks, float *__restrict__ mom1,
                       float *__restrict__ mom2) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -823,6 +828,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, FusedCfg<S, Q, DYN>::kBlocks
   if (w >= tasks) return;
   const int strip = w < edges ? -1 : (w - edges) % f.inner;
   const int part = w < edges ? w * f.per : (w - edges) / f.inner;
+  chain_wait();
   uint32_t ts1 = 0, ts2 = 0;
   if (SR) {
     const unsigned long long t = *tctr + (unsigned long long)k;

@@ -13,6 +13,7 @@
 
 #include <algorithm>
 
+#include "chain.cuh"
 #include "kernels.h"
 #include "lattice.cuh"
 #include "pairs.cuh"
@@ -32,7 +33,7 @@ constexpr int kMediumBX = 256;
 // All loads of a thread are issued before its first collision.  Plate rows
 // are block-uniform branches inside pull_node.  The stochastic-rounding
 // bits of time level t come from *tctr + k (the counter is advanced by
-// bump_kernel after a group of launches).
+// bump_kernel after a group of launches).  A chained launch (chain.cuh).
 // DYN: Knudsen number per node and step from the local pressure (the
 // medium holds 1/k_i, a.kn0 the Kn at p0).
 // MOM: also store each node's post-stream moments (rho - rho0, m_x, m_y;
@@ -40,13 +41,14 @@ constexpr int kMediumBX = 256;
 // step of the adjoint needs of the forward state.
 template <class S, bool SR, bool DYN, bool MOM = false>
 __global__ void __launch_bounds__(kStepBX)
-    step_kernel(const StepArgs a, const typename S::T *__restrict__ fin,
+    step_kernel(const StepArgs a, const typename S::T *fin,
                 typename S::T *__restrict__ fout, const float2 *__restrict__ med,
-                const unsigned long long *__restrict__ tctr, int k,
+                const unsigned long long *tctr, int k,
                 float *__restrict__ mom) {
   const int y = a.y0 + (a.rev ? (int)gridDim.y - 1 - (int)blockIdx.y : (int)blockIdx.y);
   const int xb = blockIdx.x * (kStepBX * kStepNPT) + threadIdx.x;
   const long long row = (long long)y * a.pitch;
+  chain_wait();
   float d[kStepNPT][9];
   float2 m[kStepNPT];
   float k0[kStepNPT];
@@ -102,19 +104,19 @@ cudaError_t launch_step(int storage, bool sr, const StepArgs &a, int rows, const
   __half *f16o = (__half *)fout;
   if (storage == 0) {
     if (dyn)
-      step_kernel<StoreF32, false, true><<<grid, block, 0, s>>>(a, f32i, f32o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF32, false, true>, grid, block, 0, s, a, f32i, f32o, med, tctr, k, nullptr);
     else
-      step_kernel<StoreF32, false, false><<<grid, block, 0, s>>>(a, f32i, f32o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF32, false, false>, grid, block, 0, s, a, f32i, f32o, med, tctr, k, nullptr);
   } else if (sr) {
     if (dyn)
-      step_kernel<StoreF16, true, true><<<grid, block, 0, s>>>(a, f16i, f16o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF16, true, true>, grid, block, 0, s, a, f16i, f16o, med, tctr, k, nullptr);
     else
-      step_kernel<StoreF16, true, false><<<grid, block, 0, s>>>(a, f16i, f16o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF16, true, false>, grid, block, 0, s, a, f16i, f16o, med, tctr, k, nullptr);
   } else {
     if (dyn)
-      step_kernel<StoreF16, false, true><<<grid, block, 0, s>>>(a, f16i, f16o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF16, false, true>, grid, block, 0, s, a, f16i, f16o, med, tctr, k, nullptr);
     else
-      step_kernel<StoreF16, false, false><<<grid, block, 0, s>>>(a, f16i, f16o, med, tctr, k, nullptr);
+      return launch_chained(step_kernel<StoreF16, false, false>, grid, block, 0, s, a, f16i, f16o, med, tctr, k, nullptr);
   }
   return cudaGetLastError();
 }

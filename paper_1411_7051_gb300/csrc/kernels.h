@@ -72,6 +72,20 @@ bool fused_covers(int storage, bool dyn, int nx, int ny);
 cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                          void *fout, const float2 *med, const unsigned long long *tctr, int k,
                          int nsm, cudaStream_t s);
+// Several time steps in one launch of a small lattice (tile.cuh), bit for bit
+// those of the single-step kernels: `levels` <= plan.levels steps with the
+// rounding bits from time level *tctr + k on.  tile_covers(): the lattices that
+// take it; tile_plan() picks the tiles and the steps per launch (false: none fit).
+// TilePlan: tx x ty tiles over the columns and the fluid rows.
+struct TilePlan {
+  int tx, ty, levels;
+};
+bool tile_covers(int storage, int nx, int rows);
+bool tile_plan(int storage, bool dyn, int nx, int rows, bool pressure, bool walls, int nsm,
+               TilePlan *out);
+cudaError_t launch_tile(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
+                        void *fout, const float2 *med, const unsigned long long *tctr, int k,
+                        const TilePlan &p, int levels, cudaStream_t s);
 // Store msg as the calling thread's lbmp_last_error() text.
 void set_last_error(const char *msg);
 

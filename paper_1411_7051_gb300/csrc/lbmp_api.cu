@@ -114,7 +114,6 @@ void release(lbmp_ctx *c) {
   cudaFree(c->d_flag);
   cudaFree(c->d_tctr);
   cudaFree(c->d_err);
-  cudaFree(c->d_done);
   cudaFree(c->d_hist);
   if (c->h_results) cudaFreeHost(c->h_results);
   if (c->cap_stream) cudaStreamDestroy(c->cap_stream);
@@ -174,26 +173,34 @@ cudaError_t launch_one(lbmp_ctx *c, const StepArgs &a0, const void *fin, void *f
   return lbmp::launch_step(c->p.storage, c->sr, a, c->rows(), fin, fout, c->med, c->d_tctr, k, s);
 }
 
-// Graph of `launches` launches starting from buffer `cur` (captured once
-// per medium: the launch arguments hold the storage scale), each of two steps
-// or of one, plus the counter bump when the rounding is stochastic.  A replay
-// saves the launch gaps of single launches (~3 us per step at 4096^2).
-lbmp_status get_graph(lbmp_ctx *c, cudaGraphExec_t *slot, int launches, bool two, int cur) {
+// One launch of n steps (n <= per_launch()).
+cudaError_t launch_steps(lbmp_ctx *c, const StepArgs &a, int b, int n, int k, cudaStream_t s) {
+  // (one step of an FP32 lattice: the direct kernel, which loads no halo)
+  if (c->tiled && (n > 1 || c->staged))
+    return lbmp::launch_tile(c->p.storage, c->sr, a, c->rows(), c->buf[b], c->buf[b ^ 1], c->med,
+                             c->d_tctr, k, c->tile, n, s);
+  if (n == 2 && c->fused)
+    return lbmp::launch_fused(c->p.storage, c->sr, a, c->rows(), c->buf[b], c->buf[b ^ 1], c->med,
+                              c->d_tctr, k, c->nsm, s);
+  return launch_one(c, a, c->buf[b], c->buf[b ^ 1], k, s);
+}
+
+// Graph of `launches` launches of n steps each starting from buffer `cur`
+// (captured once per medium: the launch arguments hold the storage scale), plus
+// the counter bump when the rounding is stochastic.  A replay saves the launch
+// gaps of single launches (~3 us per step at 4096^2).
+lbmp_status get_graph(lbmp_ctx *c, cudaGraphExec_t *slot, int launches, int n, int cur) {
   if (*slot) return LBMP_OK;
   StepArgs a = c->args();
   cudaGraph_t g = nullptr;
   LBMP_CK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
   int b = cur;
-  const int per = two ? 2 : 1;
   cudaError_t err = cudaSuccess;
   for (int t = 0; t < launches && err == cudaSuccess; ++t) {
-    err = two ? lbmp::launch_fused(c->p.storage, c->sr, a, c->rows(), c->buf[b], c->buf[b ^ 1],
-                                   c->med, c->d_tctr, t * per, c->nsm, c->cap_stream)
-              : launch_one(c, a, c->buf[b], c->buf[b ^ 1], t, c->cap_stream);
+    err = launch_steps(c, a, b, n, t * n, c->cap_stream);
     b ^= 1;
   }
-  if (err == cudaSuccess && c->sr)
-    err = lbmp::launch_bump(c->d_tctr, launches * per, c->cap_stream);
+  if (err == cudaSuccess && c->sr) err = lbmp::launch_bump(c->d_tctr, launches * n, c->cap_stream);
   cudaError_t end = cudaStreamEndCapture(c->cap_stream, &g);
   if (err != cudaSuccess) {
     if (g) cudaGraphDestroy(g);
@@ -360,8 +367,6 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     c->staged = p.kernel == LBMP_KERNEL_STAGED ||
                 (p.kernel == LBMP_KERNEL_AUTO && p.storage == LBMP_STORE_FP16);
     c->wide = p.kernel == LBMP_KERNEL_WIDE;
-    c->fused = p.kernel == LBMP_KERNEL_AUTO && c->drop_tile < 0 &&
-               lbmp::fused_covers(p.storage, p.kn_beta != 0.0, p.nx, p.ny);
     e = cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, c->device);
     if (e != cudaSuccess) {
       delete c;
@@ -377,6 +382,14 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     c->y_lo = (p.bc_y == LBMP_BCY_WALLS) ? 1 : 0;
     c->y_hi = (p.bc_y == LBMP_BCY_WALLS) ? p.ny - 1 : p.ny;
     c->fluid_nodes = (int64_t)p.nx * (c->y_hi - c->y_lo);
+    if (p.kernel == LBMP_KERNEL_AUTO && c->drop_tile < 0) {
+      const bool dyn = p.kn_beta != 0.0;
+      c->fused = lbmp::fused_covers(p.storage, dyn, p.nx, p.ny);
+      c->tiled = lbmp::tile_covers(p.storage, p.nx, c->rows()) &&
+                 lbmp::tile_plan(p.storage, dyn, p.nx, c->rows(), p.bc_x == LBMP_BCX_PRESSURE,
+                                 p.bc_y == LBMP_BCY_WALLS, c->nsm, &c->tile);
+      if (c->tiled) c->fused = false;
+    }
     lbmp_status st = LBMP_OK;
 #define LBMP_TRY(x)     \
   do {                  \
@@ -407,12 +420,10 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     LBMP_TRY(dalloc(c, (void **)&c->results, lbmp::kNQ * sizeof(double), "reduction results"));
     LBMP_TRY(dalloc(c, (void **)&c->d_flag, sizeof(unsigned), "validation flag"));
     LBMP_TRY(dalloc(c, (void **)&c->d_tctr, sizeof(unsigned long long), "time-level counter"));
-    LBMP_TRY(dalloc(c, (void **)&c->d_err, sizeof(unsigned), "wait error flag"));
-    e = cudaMemset(c->d_err, 0, sizeof(unsigned));
+    LBMP_TRY(dalloc(c, (void **)&c->d_err, 2 * sizeof(unsigned), "wait error flag, block counter"));
+    e = cudaMemset(c->d_err, 0, 2 * sizeof(unsigned));
     if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMemset"));
-    LBMP_TRY(dalloc(c, (void **)&c->d_done, sizeof(unsigned), "block counter"));
-    e = cudaMemset(c->d_done, 0, sizeof(unsigned));
-    if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMemset"));
+    c->d_done = c->d_err + 1;
     e = cudaMallocHost((void **)&c->h_results, (lbmp::kNQ + 1) * sizeof(double));
     if (e != cudaSuccess) LBMP_TRY(cuda_fail(e, "cudaMallocHost"));
     c->h_err = reinterpret_cast<unsigned *>(c->h_results + lbmp::kNQ);
@@ -557,14 +568,15 @@ lbmp_status lbmp_step(lbmp_ctx *c, int64_t n) {
     const DeviceScope device_scope(c->device);
     lbmp_status st = scope_status(device_scope);
     if (st) return st;
-    // launches of two steps (or one): q replays of the 32-launch graph, then
-    // one replay of each smaller power of two; an odd step at the end
-    int64_t left = c->fused ? n / 2 : n;
+    // launches of per_launch() steps: q replays of the 32-launch graph, then one
+    // replay of each smaller power of two; the steps left over in one launch
+    const int per = c->per_launch();
+    int64_t left = n / per;
     for (int level = kGraphLevels - 1; level >= 0 && left > 0; --level) {
       const int64_t size = 1ll << level;
       while (left >= size) {
         cudaGraphExec_t *slot = &c->graph[level][c->cur];
-        st = get_graph(c, slot, (int)size, c->fused, c->cur);
+        st = get_graph(c, slot, (int)size, per, c->cur);
         if (st) return st;
         LBMP_CK(cudaGraphLaunch(*slot, c->stream));
         c->launches += size + (c->sr ? 1 : 0);
@@ -573,11 +585,17 @@ lbmp_status lbmp_step(lbmp_ctx *c, int64_t n) {
         if (level < kGraphLevels - 1) break;  // one replay of each smaller size
       }
     }
-    if (c->fused && (n & 1)) {
-      cudaGraphExec_t *slot = &c->odd[c->cur];
-      st = get_graph(c, slot, 1, false, c->cur);
-      if (st) return st;
-      LBMP_CK(cudaGraphLaunch(*slot, c->stream));
+    const int rest = (int)(n % per);
+    if (rest > 0) {
+      if (c->tiled) {
+        LBMP_CK(launch_steps(c, c->args(), c->cur, rest, 0, c->stream));
+        if (c->sr) LBMP_CK(lbmp::launch_bump(c->d_tctr, rest, c->stream));
+      } else {
+        cudaGraphExec_t *slot = &c->odd[c->cur];
+        st = get_graph(c, slot, 1, 1, c->cur);
+        if (st) return st;
+        LBMP_CK(cudaGraphLaunch(*slot, c->stream));
+      }
       c->launches += 1 + (c->sr ? 1 : 0);
       c->cur ^= 1;
     }
