@@ -30,7 +30,7 @@ bool tile_plan(int storage, bool dyn, int nx, int rows, bool pressure, bool wall
                                        : TileCfg<StoreF16, false>::kNodes);
   double best = -1.0;
   for (int levels : {4, 6, 8, 12, kTileMaxLevels}) {
-    for (int tx = 1; tx == 1 || (nx / tx >= 4 && tx <= nsm); tx += 1 + tx / 12) {
+    for (int tx = 1; tx == 1 || (nx / tx >= 4 && tx <= nsm); tx += 1 + tx / 32) {
       const int tw = (nx + tx - 1) / tx, w = tw + 2 * levels;
       const int most_ty = std::min(rows, nsm / tx);
       for (int part = 4; part >= 1; --part) {  // all SMs, or three, two, one in four
