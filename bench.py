@@ -497,7 +497,7 @@ def run_ours(args, ws, rank, local):
         g3 = ws * dyn["nodes"] * K / (dyn["ms"] * 1e-3) / 1e9
         r = roofline(dyn, "StoreF32")
         r["traffic"] = r["traffic_per_update"] = r["achieved_dram"] = None  # static kernel only
-        r["kernel"] = "lbmp::step_kernel<StoreF32, false, true> (dynamic Kn)"
+        r["kernel"] += " (dynamic Kn)"
         line["fp32_dynamic_kn"] = {
             "value": g3, "unit": "GLUPS", "ms_per_step": dyn["ms"] / K,
             "what": "same workload with Kn per node and step from the local pressure "
@@ -509,11 +509,10 @@ def run_ours(args, ws, rank, local):
         g4 = ws * dyn16["nodes"] * K / (dyn16["ms"] * 1e-3) / 1e9
         r = roofline(dyn16, "StoreF16")
         r["traffic"] = r["traffic_per_update"] = r["achieved_dram"] = None
-        r["kernel"] = "lbmp::staged_step_kernel<StoreF16, SR, true> (dynamic Kn)"
+        r["kernel"] += " (dynamic Kn)"
         line["fp16_dynamic_kn"] = {
             "value": g4, "unit": "GLUPS", "ms_per_step": dyn16["ms"] / K,
-            "what": "the FP32 dynamic-Kn object with FP16-stored populations (48 B per "
-                    "update: the Kn plane at p0 staged beside the medium)",
+            "what": "the FP32 dynamic-Kn object with FP16-stored populations",
             "ratio_fp16_over_fp32": g4 / (ws * dyn["nodes"] * K / (dyn["ms"] * 1e-3) / 1e9),
             "roofline": r, "fp16_scale": dyn16["scale"], "k_g": dyn16["k_g"]}
     if adj:
@@ -548,9 +547,9 @@ def run_ours(args, ws, rank, local):
 
 # ------------------------------------------------------------------ adjoint
 # algorithmic bytes per node and time step of the backward sweep (see
-# adjoint_time()): the recompute step (the forward step's 80 plus 12 of
-# moments) and the reverse step (109.5)
-ADJOINT_RECOMPUTE_BYTES = 80 + 12
+# adjoint_time()): half a recompute launch (two steps: 36 in, 36 out, the
+# medium's 8 and two levels' moments) and the reverse step (109.5)
+ADJOINT_RECOMPUTE_BYTES = (36 + 36 + 8 + 2 * 12) / 2
 ADJOINT_REVERSE_BYTES = 36 + 12 + 8 + 16 + 36 + 48 / 32
 ADJOINT_BYTES_PER_NODE = ADJOINT_RECOMPUTE_BYTES + ADJOINT_REVERSE_BYTES
 
@@ -638,8 +637,8 @@ def adjoint_object(r, peak, peak_kind):
                          "traffic": (tr["dram_bytes_per_launch"] if tr else None),
                          "traffic_per_update": (tr["dram_bytes_per_launch"] / tr["nodes"]
                                                 if tr else None)},
-                     "kernel": "lbmp::step_kernel<StoreF32, 0, 0, 1> (recompute with moments) + "
-                               "lbmp::adjoint_step_kernel<false> (+ fold)",
+                     "kernel": "lbmp::fused_step_kernel<StoreF32> (recompute with moments) + "
+                               "lbmp::adjoint_step_kernel (+ fold)",
                      "timing": "backward sweep (recompute + reverse) = gradient minus the "
                                "forward pass, CUDA events"},
         "k_g": r["k_g"],
@@ -780,8 +779,8 @@ def batch_object(lbmp, torch, args):
     K, W = args.batch_object_steps, 10
     out = {"workload": f"batched sweep subset: {args.batch_object_media} two-component media "
                        f"(sides {list(BATCH_SIDES)}, corr. length 32) x {args.batch_kn} Kn in "
-                       "[1e-3, 10], pressure x, walls y, Forchheimer on; one launch per step "
-                       f"over all instances; median of {REPEATS} regions of {K} steps",
+                       "[1e-3, 10], pressure x, walls y, Forchheimer on; one kernel over "
+                       f"all instances; median of {REPEATS} regions of {K} steps",
            "steps": K}
     for st in ("fp16", "fp32"):
         r = batch_measure(lbmp, torch, args.batch_object_media, args.batch_kn, st, K, W,

@@ -30,9 +30,8 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
-#include <map>
-#include <tuple>
 
+#include "chain.cuh"
 #include "context.h"
 #include "device_scope.h"
 #include "kernels.h"
@@ -55,23 +54,46 @@ struct AdjArgs {
 };
 
 constexpr int kAdjBX = 128;
+constexpr int kAdjBlocks = 5;   // blocks of the reverse step on an SM
+constexpr int kAdjRows = 16;    // and the most rows that one of its warps takes
 constexpr int kFold = 32;  // reverse steps summed in FP32 before the FP64 fold
 
-// Weighted moments of an adjoint population vector.
+// The arithmetic of the reverse step rounds where it says so (fmaf, mul; a plain
+// sum is one addition), so that a kernel's form does not move its results: left to the
+// compiler, products contract one way here and another there.
+__device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
+// a b + c d, a b - c d: the second product rounded first.
+__device__ __forceinline__ float sum2(float a, float b, float c, float d) {
+  return fmaf(a, b, mul(c, d));
+}
+__device__ __forceinline__ float dif2(float a, float b, float c, float d) {
+  return fmaf(a, b, -mul(c, d));
+}
+
+// Weighted moments of an adjoint population vector.  A node's own, a pressure
+// column's and the seed's differ in the order of a few roundings.
 struct LamMom {
   float L0, Lx, Ly, Lxx, Lxy, Lyy;
 };
-__device__ __forceinline__ LamMom lam_moments(const float l[9]) {
+template <bool SEED>
+__device__ __forceinline__ LamMom lam_moments(const float l[9], bool column) {
   const float s1 = l[1] + l[3], s2 = l[2] + l[4];
   const float a57 = l[5] + l[7], a68 = l[6] + l[8];
   const float d57 = l[5] - l[7], d86 = l[8] - l[6];
+  const float diag = a57 + a68, ex = l[1] - l[3], ey = l[2] - l[4];
   LamMom M;
-  M.L0 = kW0 * l[0] + kW1 * (s1 + s2) + kW2 * (a57 + a68);
-  M.Lx = kW1 * (l[1] - l[3]) + kW2 * (d57 + d86);
-  M.Ly = kW1 * (l[2] - l[4]) + kW2 * (d57 - d86);
-  M.Lxx = kW1 * s1 + kW2 * (a57 + a68);
-  M.Lyy = kW1 * s2 + kW2 * (a57 + a68);
-  M.Lxy = kW2 * (a57 - a68);
+  const float axes = sum2(kW1, s1 + s2, kW0, l[0]);
+  M.L0 = column ? fmaf(kW2, diag, axes) : __fadd_rn(axes, mul(kW2, diag));
+  if (SEED) {
+    M.Lx = sum2(kW1, ex, kW2, d57 + d86);
+    M.Ly = sum2(kW1, ey, kW2, d57 - d86);
+  } else {
+    M.Lx = sum2(kW2, d57 + d86, kW1, ex);
+    M.Ly = sum2(kW2, d57 - d86, kW1, ey);
+  }
+  M.Lxx = sum2(kW1, s1, kW2, diag);
+  M.Lyy = sum2(kW1, s2, kW2, diag);
+  M.Lxy = mul(kW2, a57 - a68);
   return M;
 }
 
@@ -108,8 +130,8 @@ __device__ __forceinline__ Vel vel_forward(float rho, float mx, float my, float 
   }
   V.ux = V.vx * V.id;
   V.uy = V.vy * V.id;
-  V.Fx = eps * a.Gx - V.drag * V.ux;
-  V.Fy = eps * a.Gy - V.drag * V.uy;
+  V.Fx = dif2(eps, a.Gx, V.drag, V.ux);
+  V.Fy = dif2(eps, a.Gy, V.drag, V.uy);
   return V;
 }
 
@@ -119,54 +141,54 @@ struct Bar {
   float rho, mx, my, eps, lk;
 };
 
-// Reverse of vel_forward: adds to b the derivatives of ub . u + Fb . F.
+// Reverse of vel_forward: adds to b the derivatives of ub . u + Fb . F, ub
+// already without the part that F = eps G - drag u takes (- drag Fb).  FORCE: Fb is
+// not zero.
+template <bool SEED, bool FORCE>
 __device__ __forceinline__ void vel_adjoint(const Vel &V, float rho, float mx, float my,
                                             float eps, float kap, float ubx, float uby, float Fbx,
                                             float Fby, const StepArgs &a, Bar &b) {
-  // F = eps G - drag u
-  ubx -= V.drag * Fbx;
-  uby -= V.drag * Fby;
-  const float dragb = -(Fbx * V.ux + Fby * V.uy);
-  b.eps += Fbx * a.Gx + Fby * a.Gy;
+  const float dragb = FORCE ? -sum2(Fbx, V.ux, Fby, V.uy) : 0.0f;
+  if (FORCE) b.eps += sum2(Fbx, a.Gx, Fby, a.Gy);
   // u = v / den
   const float id = V.id;
-  float vbx = ubx * id, vby = uby * id;
-  float denb = -(ubx * V.ux + uby * V.uy) * id;
-  const float darcy = a.nu * eps * kap;
-  float darcyb = dragb, c0b;
+  float vbx = mul(ubx, id), vby = mul(uby, id);
+  float denb = mul(-sum2(ubx, V.ux, uby, V.uy), id);
+  const float darcy = mul(mul(a.nu, eps), kap);
+  float c0b;
   if (a.forch) {
     // drag = darcy + 2 c1 |v| / den
-    float c1b = 2.0f * dragb * V.vmag * id;
-    float vmagb = 2.0f * dragb * V.c1 * id;
-    denb -= 2.0f * dragb * V.c1 * V.vmag * id * id;
+    const float dragb_v = mul(2.0f * dragb, V.vmag), dragb_c = mul(2.0f * dragb, V.c1);
+    denb = fmaf(-mul(mul(dragb_c, V.vmag), id), id, denb);
     // den = c0 + s, s = sqrt(c0^2 + c1 |v|) >= c0 >= 1/2
     const float is = rcp_approx(V.s);
-    c0b = denb * (1.0f + V.c0 * is);
-    c1b += 0.5f * denb * V.vmag * is;
-    vmagb += 0.5f * denb * V.c1 * is;
+    c0b = mul(denb, fmaf(V.c0, is, 1.0f));
+    const float c1b = sum2(dragb_v, id, mul(0.5f * denb, V.vmag), is);
+    const float vmagb = sum2(dragb_c, id, mul(0.5f * denb, V.c1), is);
     // |v|: at v = 0 the terms it enters vanish with u, so its derivative is
     // not needed there
     if (V.vmag > 0.0f) {
       const float iv = rcp_approx(V.vmag);
-      vbx += vmagb * V.vx * iv;
-      vby += vmagb * V.vy * iv;
+      vbx = fmaf(mul(vmagb, V.vx), iv, vbx);
+      vby = fmaf(mul(vmagb, V.vy), iv, vby);
     }
     // c1 = fe_half sqrt(kap / eps): dc1/d ln k_a = -c1 / 2, dc1/d eps = -c1 / (2 eps)
-    b.lk -= 0.5f * V.c1 * c1b;
-    b.eps -= 0.5f * V.c1 * c1b * rcp_approx(eps);
+    const float h = 0.5f * V.c1;
+    b.lk = SEED ? __fadd_rn(b.lk, -mul(h, c1b)) : fmaf(-h, c1b, b.lk);
+    b.eps = fmaf(-mul(h, c1b), rcp_approx(eps), b.eps);
   } else {
     c0b = 2.0f * denb;
   }
-  darcyb += 0.25f * c0b;
   // darcy = nu eps kap: d/d ln k_a = -darcy, d/d eps = nu kap
-  b.lk -= darcy * darcyb;
-  b.eps += a.nu * kap * darcyb;
+  const float darcyb = fmaf(0.25f, c0b, dragb);
+  b.lk = fmaf(-darcy, darcyb, b.lk);
+  b.eps = fmaf(mul(a.nu, kap), darcyb, b.eps);
   // v = m / rho + eps G / 2
   const float ir = rcp_approx(rho);
-  b.mx += vbx * ir;
-  b.my += vby * ir;
-  b.rho -= (vbx * mx + vby * my) * ir * ir;
-  b.eps += 0.5f * (vbx * a.Gx + vby * a.Gy);
+  b.mx = fmaf(vbx, ir, b.mx);
+  b.my = fmaf(vby, ir, b.my);
+  b.rho = fmaf(-mul(sum2(vbx, mx, vby, my), ir), ir, b.rho);
+  b.eps = fmaf(0.5f, sum2(vbx, a.Gx, vby, a.Gy), b.eps);
 }
 
 // Adds to b the derivatives of G = sum_i lam_i g_i(rho, m; eps, k_a) of one
@@ -174,64 +196,75 @@ __device__ __forceinline__ void vel_adjoint(const Vel &V, float rho, float mx, f
 // eps] (Eq. 14) and sum_i lam_i F_i = (1 - 1/2tau) rho [3 F.L1 + (9 u.L2.F -
 // 3 (u.F) L0) / eps] (Eq. 15); eps = 0 keeps f_eq = w rho, u = 0 and
 // F = -2 m / rho.
-__device__ __forceinline__ void collide_adjoint(const float lam[9], float rho, float mx, float my,
-                                                float eps, float kap, const StepArgs &a, Bar &b) {
-  const LamMom M = lam_moments(lam);
+__device__ __forceinline__ void collide_adjoint(const float lam[9], bool column, float rho,
+                                                float mx, float my, float eps, float kap,
+                                                const StepArgs &a, Bar &b) {
+  const LamMom M = lam_moments<false>(lam, column);
   const float om = a.omega, cf = a.cforce;
   if (!(eps > 0.0f)) {
-    b.rho += om * M.L0;
-    b.mx -= 6.0f * cf * M.Lx;
-    b.my -= 6.0f * cf * M.Ly;
+    b.rho += mul(om, M.L0);
+    b.mx -= mul(6.0f * cf, M.Lx);
+    b.my -= mul(6.0f * cf, M.Ly);
     return;
   }
   const Vel V = vel_forward(rho, mx, my, eps, kap, a);
   const float ie = rcp_approx(eps);
   const float ux = V.ux, uy = V.uy, Fx = V.Fx, Fy = V.Fy;
-  const float L2ux = M.Lxx * ux + M.Lxy * uy, L2uy = M.Lxy * ux + M.Lyy * uy;
-  const float L2Fx = M.Lxx * Fx + M.Lxy * Fy, L2Fy = M.Lxy * Fx + M.Lyy * Fy;
-  const float qe = 4.5f * (ux * L2ux + uy * L2uy) - 1.5f * (ux * ux + uy * uy) * M.L0;
-  const float qf = 9.0f * (ux * L2Fx + uy * L2Fy) - 3.0f * (ux * Fx + uy * Fy) * M.L0;
-  const float Seq = M.L0 + 3.0f * (ux * M.Lx + uy * M.Ly) + qe * ie;
-  const float SF = 3.0f * (Fx * M.Lx + Fy * M.Ly) + qf * ie;
-  b.rho += om * Seq + cf * SF;
+  const float L2ux = sum2(M.Lxx, ux, M.Lxy, uy), L2uy = sum2(M.Lxy, ux, M.Lyy, uy);
+  const float L2Fx = sum2(M.Lxx, Fx, M.Lxy, Fy), L2Fy = sum2(M.Lxy, Fx, M.Lyy, Fy);
+  const float qe = dif2(4.5f, sum2(ux, L2ux, uy, L2uy), mul(1.5f, sum2(ux, ux, uy, uy)), M.L0);
+  const float qf = dif2(9.0f, sum2(ux, L2Fx, uy, L2Fy), mul(3.0f, sum2(ux, Fx, uy, Fy)), M.L0);
+  const float Seq = fmaf(qe, ie, fmaf(3.0f, sum2(ux, M.Lx, uy, M.Ly), M.L0));
+  const float SF = sum2(3.0f, sum2(Fx, M.Lx, Fy, M.Ly), qf, ie);
+  b.rho += sum2(om, Seq, cf, SF);
   // dSeq/du = dSF/dF
-  const float ax = 3.0f * M.Lx + (9.0f * L2ux - 3.0f * ux * M.L0) * ie;
-  const float ay = 3.0f * M.Ly + (9.0f * L2uy - 3.0f * uy * M.L0) * ie;
-  const float ubx = rho * (om * ax + cf * (9.0f * L2Fx - 3.0f * Fx * M.L0) * ie);
-  const float uby = rho * (om * ay + cf * (9.0f * L2Fy - 3.0f * Fy * M.L0) * ie);
-  b.eps -= rho * (om * qe + cf * qf) * ie * ie;
-  vel_adjoint(V, rho, mx, my, eps, kap, ubx, uby, rho * cf * ax, rho * cf * ay, a, b);
+  const float ax = sum2(3.0f, M.Lx, dif2(9.0f, L2ux, mul(3.0f, ux), M.L0), ie);
+  const float ay = sum2(3.0f, M.Ly, dif2(9.0f, L2uy, mul(3.0f, uy), M.L0), ie);
+  const float ubx = sum2(om, ax, mul(cf, dif2(9.0f, L2Fx, mul(3.0f, Fx), M.L0)), ie);
+  const float uby = sum2(om, ay, mul(cf, dif2(9.0f, L2Fy, mul(3.0f, Fy), M.L0)), ie);
+  b.eps -= mul(mul(mul(rho, sum2(om, qe, cf, qf)), ie), ie);
+  const float rcf = mul(rho, cf), Fbx = mul(rcf, ax), Fby = mul(rcf, ay);
+  vel_adjoint<false, true>(V, rho, mx, my, eps, kap, dif2(rho, ubx, V.drag, Fbx),
+                         dif2(rho, uby, V.drag, Fby), Fbx, Fby, a, b);
 }
 
 // Pressure column b next to interior node n: f_b = f_n + f_eq(rho_b, u_n;
 // eps_b) - f_eq(rho_n, u_n; eps_n).  Adds to bn the derivatives of
 // sum_i lb_i f_b,i with respect to n's moments and parameters (the identity
 // part, lb itself, is added by the caller) and to eb the one of eps_b.
+template <bool SEED>
 __device__ __forceinline__ void neep_adjoint(const float lb[9], float rho_n, float mx, float my,
                                              float eps_n, float kap_n, float eps_b, float rho_b,
                                              const StepArgs &a, Bar &bn, float &eb) {
-  const LamMom M = lam_moments(lb);
+  const LamMom M = lam_moments<SEED>(lb, true);
   if (!(eps_n > 0.0f)) {  // u_n = 0: f_b = f_n + w (rho_b - rho_n)
     bn.rho -= M.L0;
     return;
   }
   const Vel V = vel_forward(rho_n, mx, my, eps_n, kap_n, a);
   const float ux = V.ux, uy = V.uy;
-  const float L2ux = M.Lxx * ux + M.Lxy * uy, L2uy = M.Lxy * ux + M.Lyy * uy;
-  const float q = 4.5f * (ux * L2ux + uy * L2uy) - 1.5f * (ux * ux + uy * uy) * M.L0;
-  const float cx = 3.0f * M.Lx, cy = 3.0f * M.Ly;
-  const float qx = 9.0f * L2ux - 3.0f * ux * M.L0, qy = 9.0f * L2uy - 3.0f * uy * M.L0;
+  const float L2ux = sum2(M.Lxx, ux, M.Lxy, uy), L2uy = sum2(M.Lxy, ux, M.Lyy, uy);
+  const float q = dif2(4.5f, sum2(ux, L2ux, uy, L2uy), mul(1.5f, sum2(ux, ux, uy, uy)), M.L0);
+  const float cx = mul(3.0f, M.Lx), cy = mul(3.0f, M.Ly);
+  const float qx = dif2(9.0f, L2ux, mul(3.0f, ux), M.L0);
+  const float qy = dif2(9.0f, L2uy, mul(3.0f, uy), M.L0);
+  // d/du of sum_i lb_i f_eq_i / rho at porosity eps: c + q / eps
   const float ien = rcp_approx(eps_n);
-  bn.rho -= M.L0 + (ux * cx + uy * cy) + q * ien;
-  float ubx = -rho_n * (cx + qx * ien), uby = -rho_n * (cy + qy * ien);
-  bn.eps += rho_n * q * ien * ien;
+  const bool open = !SEED && eps_b > 0.0f;
+  bn.rho -= fmaf(q, ien, __fadd_rn(M.L0, sum2(ux, cx, uy, cy)));
+  const float dux = open ? sum2(3.0f, M.Lx, qx, ien) : fmaf(qx, ien, cx);
+  const float duy = open ? sum2(3.0f, M.Ly, qy, ien) : fmaf(qy, ien, cy);
+  float ubx = mul(-rho_n, dux), uby = mul(-rho_n, duy);
+  bn.eps = fmaf(mul(mul(rho_n, q), ien), ien, bn.eps);
   if (eps_b > 0.0f) {
     const float ieb = rcp_approx(eps_b);
-    ubx += rho_b * (cx + qx * ieb);
-    uby += rho_b * (cy + qy * ieb);
-    eb -= rho_b * q * ieb * ieb;
+    ubx = sum2(-rho_n, dux, rho_b,
+               open ? sum2(3.0f, M.Lx, qx, ieb) : fmaf(qx, ieb, cx));
+    uby = sum2(-rho_n, duy, rho_b,
+               open ? sum2(3.0f, M.Ly, qy, ieb) : fmaf(qy, ieb, cy));
+    eb -= mul(mul(mul(rho_b, q), ieb), ieb);
   }
-  vel_adjoint(V, rho_n, mx, my, eps_n, kap_n, ubx, uby, 0.0f, 0.0f, a, bn);
+  vel_adjoint<SEED, false>(V, rho_n, mx, my, eps_n, kap_n, ubx, uby, 0.0f, 0.0f, a, bn);
 }
 
 __device__ __forceinline__ float lam_at(const AdjArgs &A, int i, int x, int y) {
@@ -276,15 +309,12 @@ __device__ __forceinline__ void moments(const float d[9], float rho0, float &rho
   my = (d[2] - d[4]) + ((d[5] - d[7]) + (d[6] - d[8]));
 }
 
-// Adjoint of the pressure column beside interior node (x, y), formed and
-// pushed into the node by the node's own thread: the column's adjoint lb =
-// (1 - 1/tau) lambda*_b + its collision adjoint (SEED: the objective's
-// dJ/df_b instead), then E^T.  Adds lb to mu and the node's moment and
-// parameter sensitivities to bn; writes the column's parameter gradients.
-template <bool SEED>
-__device__ __forceinline__ void column_adjoint(const AdjArgs &A, int x, int y, float rho,
-                                               float mx, float my, float2 mn, float mu[9],
-                                               Bar &bn) {
+// The objective's adjoint of the pressure column beside interior node (x, y),
+// formed and pushed into the node by the node's own thread (E^T): adds it to mu and
+// the node's moment and parameter sensitivities to bn; writes the column's
+// parameter gradients.
+__device__ __forceinline__ void column_seed(const AdjArgs &A, int x, int y, float rho, float mx,
+                                            float my, float2 mn, float mu[9], Bar &bn) {
   const StepArgs &a = A.a;
   const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
@@ -295,36 +325,20 @@ __device__ __forceinline__ void column_adjoint(const AdjArgs &A, int x, int y, f
     const int xb = side ? a.nx - 1 : 0;
     const long long jb = (long long)y * a.pitch + xb;
     const float2 mb = A.med[jb];
-    float rb, mbx, mby;
-    if (SEED) {
-      float fb[9];
-      pressure_node<StoreF32>(A.fin, A.med, a, xb, y, mb.x, fb);
-      moments(fb, a.rho0, rb, mbx, mby);
-    } else {  // the column's moments as its forward step stored them
-      rb = a.rho0 + A.mom[jb];
-      mbx = A.mom[a.plane + jb];
-      mby = A.mom[2 * a.plane + jb];
-    }
+    float rb, mbx, mby, fb[9];
+    pressure_node<StoreF32>(A.fin, A.med, a, xb, y, mb.x, fb);
+    moments(fb, a.rho0, rb, mbx, mby);
     Bar bb = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-    float lb[9];
-    if (SEED) {
-      if (mb.x > 0.0f) {
-        const Vel V = vel_forward(rb, mbx, mby, mb.x, mb.y, a);
-        vel_adjoint(V, rb, mbx, mby, mb.x, mb.y, A.coef, 0.0f, 0.0f, 0.0f, a, bb);
-      }
-#pragma unroll
-      for (int i = 0; i < 9; ++i) lb[i] = bb.rho + ex[i] * bb.mx + ey[i] * bb.my;
-    } else {
-      float lpb[9];
-      reverse_pull(A, xb, y, lpb);
-      collide_adjoint(lpb, rb, mbx, mby, mb.x, mb.y, a, bb);
-#pragma unroll
-      for (int i = 0; i < 9; ++i)
-        lb[i] = fmaf(a.one_m_omega, lpb[i], bb.rho + ex[i] * bb.mx + ey[i] * bb.my);
+    if (mb.x > 0.0f) {
+      const Vel V = vel_forward(rb, mbx, mby, mb.x, mb.y, a);
+      vel_adjoint<true, false>(V, rb, mbx, mby, mb.x, mb.y, A.coef, 0.0f, 0.0f, 0.0f, a, bb);
     }
+    float lb[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) lb[i] = bb.rho + ex[i] * bb.mx + ey[i] * bb.my;
     float eb = 0.0f;
     const float rho_b = a.rho0 + (side ? a.drho_out : a.drho_in);
-    neep_adjoint(lb, rho, mx, my, mn.x, mn.y, mb.x, rho_b, a, bn, eb);
+    neep_adjoint<true>(lb, rho, mx, my, mn.x, mn.y, mb.x, rho_b, a, bn, eb);
 #pragma unroll
     for (int i = 0; i < 9; ++i) mu[i] += lb[i];
     const float2 g = A.acc[jb];  // only this thread touches the column node
@@ -332,11 +346,9 @@ __device__ __forceinline__ void column_adjoint(const AdjArgs &A, int x, int y, f
   }
 }
 
-// One reverse step over the fluid rows: mu^t from mu^{t+1} and f^t.
-// SEED: the objective instead, mu^N = dJ/df^N.  Pressure-column threads
-// return at once (their neighbours handle them).
-template <bool SEED>
-__global__ void __launch_bounds__(kAdjBX, 8) adjoint_step_kernel(const AdjArgs A) {
+// The objective's seed, mu^N = dJ/df^N.  Pressure-column threads return at
+// once (their neighbours handle them).
+__global__ void __launch_bounds__(kAdjBX, 8) adjoint_seed_kernel(const AdjArgs A) {
   const StepArgs &a = A.a;
   const int y = a.y0 + blockIdx.y;
   const int x = blockIdx.x * kAdjBX + threadIdx.x;
@@ -345,59 +357,183 @@ __global__ void __launch_bounds__(kAdjBX, 8) adjoint_step_kernel(const AdjArgs A
   const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
   const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
   const long long j = (long long)y * a.pitch + x;
-  // the accumulators are read up front so that their latency overlaps the
-  // population loads
   const float2 g0 = A.acc[j];
   const float2 m = __ldg(A.med + j);
-  float mu[9];
+  float mu[9], d[9];
   float rho, mx, my;
-  if (SEED) {
-    float d[9];
-    pull_node<StoreF32>(A.fin, a, x, y, d);
-    moments(d, a.rho0, rho, mx, my);
-  } else {  // the moments of f^t, stored by the recompute step (bit for bit
-            // the sums above)
-    rho = a.rho0 + A.mom[j];
-    mx = A.mom[a.plane + j];
-    my = A.mom[2 * a.plane + j];
-  }
+  pull_node<StoreF32>(A.fin, a, x, y, d);
+  moments(d, a.rho0, rho, mx, my);
   Bar b = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
-  if (SEED) {
-    if (m.x > 0.0f) {
-      const Vel V = vel_forward(rho, mx, my, m.x, m.y, a);
-      vel_adjoint(V, rho, mx, my, m.x, m.y, A.coef, 0.0f, 0.0f, 0.0f, a, b);
-    }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) mu[i] = 0.0f;
-  } else {
-    float lp[9];
-    // Away from the lattice edges every destination z + e_i is a plain fluid
-    // node at a fixed offset; the edge rules of reverse_pull apply to the rest.
-    const bool inner = x >= 2 && x <= a.nx - 3 && y >= 2 && y <= a.ny - 3;
-    if (inner) {
-      const float *l = A.lam_in + j;
-      const long long P = a.plane, R = a.pitch;
-      lp[0] = l[0];
-      lp[1] = l[P + 1];
-      lp[2] = l[2 * P + R];
-      lp[3] = l[3 * P - 1];
-      lp[4] = l[4 * P - R];
-      lp[5] = l[5 * P + R + 1];
-      lp[6] = l[6 * P + R - 1];
-      lp[7] = l[7 * P - R - 1];
-      lp[8] = l[8 * P - R + 1];
-    } else {
-      reverse_pull(A, x, y, lp);
-    }
-    collide_adjoint(lp, rho, mx, my, m.x, m.y, a, b);
-#pragma unroll
-    for (int i = 0; i < 9; ++i) mu[i] = a.one_m_omega * lp[i];
+  if (m.x > 0.0f) {
+    const Vel V = vel_forward(rho, mx, my, m.x, m.y, a);
+    vel_adjoint<true, false>(V, rho, mx, my, m.x, m.y, A.coef, 0.0f, 0.0f, 0.0f, a, b);
   }
-  if (a.pressure && (x == 1 || x == a.nx - 2)) column_adjoint<SEED>(A, x, y, rho, mx, my, m, mu, b);
+#pragma unroll
+  for (int i = 0; i < 9; ++i) mu[i] = 0.0f;
+  if (a.pressure && (x == 1 || x == a.nx - 2)) column_seed(A, x, y, rho, mx, my, m, mu, b);
 #pragma unroll
   for (int i = 0; i < 9; ++i)
     A.lam_out[i * a.plane + j] = mu[i] + b.rho + ex[i] * b.mx + ey[i] * b.my;
   A.acc[j] = make_float2(g0.x + b.eps, g0.y + b.lk);
+}
+
+// What a reverse step reads of one node.
+struct RevIn {
+  float l[9], r, mx, my;
+  float2 med, acc;
+};
+__device__ __forceinline__ void rev_fields(const AdjArgs &A, long long j, RevIn &n) {
+  n.med = __ldg(A.med + j);
+  n.acc = A.acc[j];
+  n.r = A.mom[j];
+  n.mx = A.mom[A.a.plane + j];
+  n.my = A.mom[2 * A.a.plane + j];
+}
+__device__ __forceinline__ void rev_store(const AdjArgs &A, long long j, const float mu[9],
+                                          const Bar &b, float2 acc) {
+  const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+  const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+#pragma unroll
+  for (int i = 0; i < 9; ++i) {
+    float s = __fadd_rn(mu[i], b.rho);
+    if (ex[i]) s = __fadd_rn(s, ex[i] > 0 ? b.mx : -b.mx);
+    if (ey[i]) s = __fadd_rn(s, ey[i] > 0 ? b.my : -b.my);
+    A.lam_out[i * A.a.plane + j] = s;
+  }
+  A.acc[j] = make_float2(acc.x + b.eps, acc.y + b.lk);
+}
+
+// The nodes next to the pressure columns and, through them, the columns: four
+// lanes a node, one for the node itself and one for each column beside it, so
+// that their collision adjoints run at the same time (64 x 64, 400 steps: 4.6 ms
+// with one lane that takes them in turn, 3.6 with one each).  The column's
+// adjoint, (1 - 1/tau) lambda*_b + its collision adjoint, then goes to the node's
+// lane (E^T).  A lane's loads are a row apart: few nodes a warp spread them.
+__device__ __forceinline__ void edge_nodes(const AdjArgs &A, int t, int rows) {
+  const StepArgs &a = A.a;
+  const int role = t & 3, node = t >> 2, side = node >= rows;
+  const int xn = side ? a.nx - 2 : 1;
+  const int x = role == 0 ? xn : role == 1 ? 0 : a.nx - 1;
+  const bool live = node < (a.nx == 3 ? rows : 2 * rows) &&
+                    (role == 0 || (role == 1 && xn == 1) || (role == 2 && xn == a.nx - 2));
+  const int y = a.y0 + (live ? node - side * rows : 0);
+  const long long j = (long long)y * a.pitch + x;
+  RevIn n = {};
+  Bar b = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+  float v[9] = {};
+  float rho = 1.0f;
+  if (live) {
+    rev_fields(A, j, n);
+    reverse_pull(A, x, y, n.l);
+    rho = a.rho0 + n.r;
+    collide_adjoint(n.l, role != 0, rho, n.mx, n.my, n.med.x, n.med.y, a, b);
+    if (role == 0) {
+#pragma unroll
+      for (int i = 0; i < 9; ++i) v[i] = mul(a.one_m_omega, n.l[i]);
+    } else {
+      const int ex[9] = {0, 1, 0, -1, 0, 1, -1, -1, 1};
+      const int ey[9] = {0, 0, 1, 0, -1, 1, 1, -1, -1};
+#pragma unroll
+      for (int i = 0; i < 9; ++i)
+        v[i] = fmaf(a.one_m_omega, n.l[i], b.rho + ex[i] * b.mx + ey[i] * b.my);
+    }
+  }
+#pragma unroll 1
+  for (int k = 1; k <= 2; ++k) {
+    float lb[9], eb = 0.0f;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) lb[i] = __shfl_sync(0xffffffffu, v[i], k, 4);
+    const float eps_b = __shfl_sync(0xffffffffu, n.med.x, k, 4);
+    if (live && role == 0 && xn == (k == 1 ? 1 : a.nx - 2)) {
+      const float rho_b = a.rho0 + (k == 1 ? a.drho_in : a.drho_out);
+      neep_adjoint<false>(lb, rho, n.mx, n.my, n.med.x, n.med.y, eps_b, rho_b, a, b, eb);
+#pragma unroll
+      for (int i = 0; i < 9; ++i) v[i] += lb[i];
+    }
+    eb = __shfl_sync(0xffffffffu, eb, 0, 4);
+    if (role == k) b.eps += eb;
+  }
+  if (!live) return;
+  if (role == 0)
+    rev_store(A, j, v, b, n.acc);
+  else
+    A.acc[j] = make_float2(n.acc.x + b.eps, n.acc.y + b.lk);
+}
+
+// One reverse step over the fluid rows: mu^t from mu^{t+1} and f^t.  The first
+// `edges` blocks take the nodes next to pressure columns (and through them the
+// columns); each further warp takes 32 columns of `seg` rows, upwards in y.
+//
+// 108 B a node (mu in and out, moments, medium, accumulators) against some 400
+// instructions.  With a thread per node it waited for its loads at 54 % of the issue
+// slots, and the warps at a pressure column computed three nodes in turn: 26 us
+// at 1024^2.  Walking the rows with the next row's 16 values in flight while
+// one is computed: 18 us, 6.3 TB/s.  Five blocks of 85 registers an SM (four: +1.9 us,
+// six: the same).
+__global__ void __launch_bounds__(kAdjBX, kAdjBlocks)
+    adjoint_step_kernel(const AdjArgs A, int rows, int edges, int strips, int seg) {
+  chain_wait();
+  const StepArgs &a = A.a;
+  if ((int)blockIdx.x < edges) {
+    edge_nodes(A, blockIdx.x * kAdjBX + threadIdx.x, rows);
+    return;
+  }
+  const int task = (blockIdx.x - edges) * (kAdjBX / 32) + threadIdx.x / 32;
+  const int part = task / strips;
+  const int x = (task - part * strips) * 32 + (threadIdx.x & 31);
+  int y = a.y0 + part * seg;
+  const int end = min(y + seg, a.y0 + rows);
+  if (y >= end || x >= a.nx) return;
+  if (a.pressure && (x < 2 || x > a.nx - 3)) return;
+  const int west = x > 0 ? -1 : a.nx - 1, east = x < a.nx - 1 ? 1 : 1 - a.nx;
+  auto load = [&](int y, RevIn &n) {
+    const long long j = (long long)y * a.pitch + x;
+    rev_fields(A, j, n);
+    if (a.walls && (y == 1 || y == a.ny - 2)) {
+      reverse_pull(A, x, y, n.l);
+      return;
+    }
+    const int up = (y < a.ny - 1 ? 1 : 1 - a.ny) * a.pitch, down = (y > 0 ? -1 : a.ny - 1) * a.pitch;
+    const float *l = A.lam_in + j;
+    const long long P = a.plane;
+    n.l[0] = l[0];
+    n.l[1] = l[P + east];
+    n.l[2] = l[2 * P + up];
+    n.l[3] = l[3 * P + west];
+    n.l[4] = l[4 * P + down];
+    n.l[5] = l[5 * P + up + east];
+    n.l[6] = l[6 * P + up + west];
+    n.l[7] = l[7 * P + down + west];
+    n.l[8] = l[8 * P + down + east];
+  };
+  RevIn n;
+  load(y, n);
+  for (; y < end; ++y) {
+    RevIn next = n;
+    if (y + 1 < end) load(y + 1, next);
+    const float rho = a.rho0 + n.r;
+    Bar b = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    collide_adjoint(n.l, false, rho, n.mx, n.my, n.med.x, n.med.y, a, b);
+    float mu[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) mu[i] = mul(a.one_m_omega, n.l[i]);
+    rev_store(A, (long long)y * a.pitch + x, mu, b, n.acc);
+    n = next;
+  }
+}
+
+// Rows a warp: what fills the chip once beside the edge blocks, at most 16 (8: +1.6 us
+// a step at 1024^2, 32: the same).
+static cudaError_t launch_adjoint_step(const AdjArgs &A, int rows, int nsm, cudaStream_t s) {
+  constexpr int kWarps = kAdjBX / 32;
+  const int edges = A.a.pressure ? (8 * rows + kAdjBX - 1) / kAdjBX : 0;  // edge_nodes()
+  const int strips = (A.a.nx + 31) / 32;
+  const int slots = std::max(nsm * kAdjBlocks - edges, nsm) * kWarps;
+  const int parts = std::max(1, slots / strips);
+  const int seg = std::min((rows + parts - 1) / parts, kAdjRows);
+  const int tasks = strips * ((rows + seg - 1) / seg);
+  return launch_chained(adjoint_step_kernel, dim3(edges + (tasks + kWarps - 1) / kWarps),
+                        dim3(kAdjBX), 0, s, A, rows, edges, strips, seg);
 }
 
 // Folds the FP32 accumulators of the fluid rows into the FP64 gradients
@@ -406,6 +542,7 @@ __global__ void __launch_bounds__(kAdjBX) adjoint_fold_kernel(const AdjArgs A) {
   const StepArgs &a = A.a;
   const int y = a.y0 + blockIdx.y;
   const int x = blockIdx.x * kAdjBX + threadIdx.x;
+  chain_wait();
   if (x >= a.nx) return;
   const long long j = (long long)y * a.pitch + x;
   const float2 g = A.acc[j];
@@ -465,22 +602,38 @@ struct DevBuf {
     }                                                                                    \
   } while (0)
 
-// The launches of one backward segment: n recompute steps from the
-// checkpoint copy in seg[0] (the two state buffers alternate; level t's
-// moments go to mom + t * mom_level), then the n reverse steps from the
-// last level down, with an FP64 fold after every kFold-th reverse step of
-// the whole sweep (`reversed` of them done before this segment).  lam[0]
-// holds Lambda^{t+1} of the segment's last level on entry.
-cudaError_t enqueue_segment(const lbmp::AdjArgs &A0, int rows, const float2 *med, char *segp,
-                            size_t state, char *momp, size_t mom_level, int64_t n,
-                            float *const lam[2], int64_t reversed, cudaStream_t s) {
+// The launches of one backward segment: n recompute steps from checkpoint ck
+// (the first step reads it in place, the two state buffers at segp then
+// alternate; level t's moments go to mom + t * mom_level; two steps per launch
+// on the lattices where that is the faster form), then the n reverse steps from
+// the last level down, with an FP64 fold after every kFold-th reverse step of the
+// whole sweep (`reversed` of them done before this segment).  lam[0] holds
+// Lambda^{t+1} of the segment's last level on entry.  Adds its launches to
+// *launches.
+cudaError_t enqueue_segment(const lbmp::AdjArgs &A0, int rows, const float2 *med, const char *ck,
+                            char *segp, size_t state, char *momp, size_t mom_level, int64_t n,
+                            float *const lam[2], int64_t reversed, int nsm, int64_t *launches,
+                            cudaStream_t s) {
   lbmp::AdjArgs A = A0;
   const lbmp::StepArgs &a = A.a;
+  const bool pairs = lbmp::fused_covers(LBMP_STORE_FP32, false, a.nx, a.ny);
   cudaError_t e = cudaSuccess;
-  for (int64_t t = 0; t < n && e == cudaSuccess; ++t)
-    e = lbmp::launch_step_moments(a, rows, (const float *)(segp + state * (t & 1)),
-                                  (float *)(segp + state * ((t + 1) & 1)), med,
-                                  (float *)(momp + mom_level * t), s);
+  const float *in = (const float *)ck;
+  int to = 0;
+  for (int64_t t = 0; t < n && e == cudaSuccess;) {
+    float *out = (float *)(segp + state * to);
+    float *m0 = (float *)(momp + mom_level * t), *m1 = (float *)(momp + mom_level * (t + 1));
+    if (pairs && t + 1 < n) {
+      e = lbmp::launch_fused_moments(a, rows, in, out, med, m0, m1, nsm, s);
+      t += 2;
+    } else {
+      e = lbmp::launch_step_moments(a, rows, in, out, med, m0, s);
+      t += 1;
+    }
+    ++*launches;
+    in = out;
+    to ^= 1;
+  }
   const dim3 blk(lbmp::kAdjBX), grd((a.nx + lbmp::kAdjBX - 1) / lbmp::kAdjBX, rows);
   int next = 0;
   for (int64_t t = n - 1; t >= 0 && e == cudaSuccess; --t) {
@@ -488,27 +641,16 @@ cudaError_t enqueue_segment(const lbmp::AdjArgs &A0, int rows, const float2 *med
     A.lam_out = lam[next ^ 1];
     A.fin = nullptr;
     A.mom = (const float *)(momp + mom_level * t);
-    lbmp::adjoint_step_kernel<false><<<grd, blk, 0, s>>>(A);
-    e = cudaGetLastError();
+    e = lbmp::launch_adjoint_step(A, rows, nsm, s);
+    ++*launches;
     next ^= 1;
     if (e == cudaSuccess && ++reversed % lbmp::kFold == 0) {
-      lbmp::adjoint_fold_kernel<<<grd, blk, 0, s>>>(A);
-      e = cudaGetLastError();
+      e = lbmp::launch_chained(lbmp::adjoint_fold_kernel, grd, blk, 0, s, A);
+      ++*launches;
     }
   }
   return e;
 }
-
-// Instantiated backward-segment graphs of one gradient call, keyed by the
-// segment length, which adjoint buffer holds Lambda^{t+1} on entry, and
-// the fold phase (reversed steps mod kFold): full segments share one graph
-// per phase, so a call captures at most kFold + 1 of them.
-struct SegmentGraphs {
-  std::map<std::tuple<int64_t, int, int>, cudaGraphExec_t> g;
-  ~SegmentGraphs() {
-    for (auto &kv : g) cudaGraphExecDestroy(kv.second);
-  }
-};
 
 }  // namespace
 
@@ -539,23 +681,24 @@ extern "C" lbmp_status lbmp_permeability_gradient(lbmp_ctx *c, int64_t nsteps, i
     const size_t state = c->buf_bytes();
     const size_t field = (size_t)c->plane * sizeof(double);
     cudaStream_t s = c->stream;
-    // checkpoints (one per segment), two states for the recompute, the
+    // one allocation (one of each: 0.6 ms more at 1024^2 and 400 steps) for
+    // the checkpoints (one per segment), two states for the recompute, the
     // moments of the levels of one segment, the two adjoint levels, the FP64
-    // gradient fields
+    // gradient fields with the accumulators
     const size_t mom_level = (size_t)c->plane * 3 * sizeof(float);
-    DevBuf ck, seg, mom, lam, grad, outs;
-    ACK(cudaMalloc(&ck.p, state * (size_t)nseg));
-    ACK(cudaMalloc(&seg.p, state * 2));
-    ACK(cudaMalloc(&mom.p, mom_level * (size_t)every));
-    ACK(cudaMalloc(&lam.p, state * 2));
-    const size_t accb = (size_t)c->plane * sizeof(float2);
-    ACK(cudaMalloc(&grad.p, field * 2 + accb));
-    ACK(cudaMemsetAsync(lam.p, 0, state * 2, s));
-    ACK(cudaMemsetAsync(grad.p, 0, field * 2 + accb, s));
-    char *ckp = (char *)ck.p, *segp = (char *)seg.p, *momp = (char *)mom.p;
-    float *lam0 = (float *)lam.p, *lam1 = (float *)((char *)lam.p + state);
-    double *g_eps = (double *)grad.p, *g_lk = (double *)((char *)grad.p + field);
-    float2 *acc = (float2 *)((char *)grad.p + 2 * field);
+    const size_t grad_bytes = 2 * field + (size_t)c->plane * sizeof(float2);
+    const size_t sizes[5] = {state * (size_t)nseg, state * 2, mom_level * (size_t)every, state * 2,
+                             grad_bytes};
+    size_t at[6] = {0};
+    for (int k = 0; k < 5; ++k) at[k + 1] = at[k] + (sizes[k] + 511) / 512 * 512;
+    DevBuf work, outs;
+    ACK(cudaMalloc(&work.p, at[5]));
+    char *base = (char *)work.p;
+    char *ckp = base, *segp = base + at[1], *momp = base + at[2];
+    ACK(cudaMemsetAsync(base + at[3], 0, at[5] - at[3], s));
+    float *lam0 = (float *)(base + at[3]), *lam1 = (float *)(base + at[3] + state);
+    double *g_eps = (double *)(base + at[4]), *g_lk = (double *)(base + at[4] + field);
+    float2 *acc = (float2 *)(base + at[4] + 2 * field);
 
     // forward pass from rest in the context's own buffers (the step graphs
     // of lbmp_step), checkpointing the first level of every segment
@@ -595,38 +738,19 @@ extern "C" lbmp_status lbmp_permeability_gradient(lbmp_ctx *c, int64_t nsteps, i
     A.mom = nullptr;
     A.lam_in = lam1;
     A.lam_out = lam0;
-    lbmp::adjoint_step_kernel<true><<<grd, blk, 0, s>>>(A);
+    lbmp::adjoint_seed_kernel<<<grd, blk, 0, s>>>(A);
     ACK(cudaGetLastError());
     // backward, one segment at a time: recompute its levels from the
     // checkpoint (keeping only their moments), then run the reverse steps
-    // over them; each segment replays a captured graph
+    // over them.  The launches go straight into the stream: a graph of a segment
+    // (one per fold phase) was captured and instantiated to be replayed a few
+    // times (64 x 64, 400 steps: 4.46 ms against 3.73).
     float *lams[2] = {lam0, lam1};  // lams[0]: Lambda^{t+1} of the next reverse step
     int64_t reversed = 0;          // the FP32 accumulators fold every kFold reverse steps
-    SegmentGraphs graphs;
     for (int64_t sg = nseg - 1; sg >= 0; --sg) {
       const int64_t t0 = sg * every, n = std::min(every, nsteps - t0);
-      ACK(cudaMemcpyAsync(segp, ckp + state * sg, state, cudaMemcpyDeviceToDevice, s));
-      const auto key = std::make_tuple(n, lams[0] == lam0 ? 0 : 1, (int)(reversed % lbmp::kFold));
-      auto it = graphs.g.find(key);
-      if (it == graphs.g.end()) {
-        cudaGraph_t g = nullptr;
-        ACK(cudaStreamBeginCapture(c->cap_stream, cudaStreamCaptureModeThreadLocal));
-        cudaError_t ce = enqueue_segment(A, rows, c->med, segp, state, momp, mom_level, n, lams,
-                                         reversed, c->cap_stream);
-        cudaError_t ee = cudaStreamEndCapture(c->cap_stream, &g);
-        if (ce != cudaSuccess || ee != cudaSuccess) {
-          if (g) cudaGraphDestroy(g);
-          ACK(ce != cudaSuccess ? ce : ee);
-        }
-        cudaGraphExec_t exec = nullptr;
-        cudaError_t ie = cudaGraphInstantiate(&exec, g, 0);
-        cudaGraphDestroy(g);
-        ACK(ie);
-        it = graphs.g.emplace(key, exec).first;
-      }
-      ACK(cudaGraphLaunch(it->second, s));
-      const int64_t folds = (reversed + n) / lbmp::kFold - reversed / lbmp::kFold;
-      c->launches += 2 * n + folds;
+      ACK(enqueue_segment(A, rows, c->med, ckp + state * sg, segp, state, momp, mom_level, n, lams,
+                          reversed, c->nsm, &c->launches, s));
       reversed += n;
       if (n & 1) std::swap(lams[0], lams[1]);
     }

@@ -90,4 +90,11 @@ cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, cons
 #undef LBMP_FUSED
 }
 
+cudaError_t launch_fused_moments(const StepArgs &a, int rows, const float *fin, float *fout,
+                                 const float2 *med, float *mom1, float *mom2, int nsm,
+                                 cudaStream_t s) {
+  return launch_fused_t<StoreF32, false, false, true>(a, rows, fin, fout, med, nullptr, 0, nsm,
+                                                      mom1, mom2, s);
+}
+
 }  // namespace lbmp

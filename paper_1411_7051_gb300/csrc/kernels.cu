@@ -126,9 +126,8 @@ cudaError_t launch_step_moments(const StepArgs &a, int rows, const float *fin, f
   if (rows <= 0 || a.nx <= 0) return cudaSuccess;
   dim3 block(kStepBX);
   dim3 grid((a.nx + kStepBX * kStepNPT - 1) / (kStepBX * kStepNPT), rows);
-  step_kernel<StoreF32, false, false, true><<<grid, block, 0, s>>>(a, fin, fout, med, nullptr, 0,
-                                                                   mom);
-  return cudaGetLastError();
+  return launch_chained(step_kernel<StoreF32, false, false, true>, grid, block, 0, s, a, fin, fout,
+                        med, nullptr, 0, mom);
 }
 
 // -------------------------------------------------------- wide variant

@@ -52,6 +52,11 @@ cudaError_t launch_step(int storage, bool sr, const StepArgs &a, int rows, const
 // three [ny][pitch] float planes at mom, a.plane apart (adjoint recompute).
 cudaError_t launch_step_moments(const StepArgs &a, int rows, const float *fin, float *fout,
                                 const float2 *med, float *mom, cudaStream_t s);
+// Two such steps in one launch (fused.cuh): the moments of the two levels go
+// to mom1 and mom2.
+cudaError_t launch_fused_moments(const StepArgs &a, int rows, const float *fin, float *fout,
+                                 const float2 *med, float *mom1, float *mom2, int nsm,
+                                 cudaStream_t s);
 // Vectorised FP16 variant of the same step (four nodes per thread).
 cudaError_t launch_wide(bool sr, const StepArgs &a, int rows, const void *fin, void *fout,
                         const float2 *med, const unsigned long long *tctr, int k,

@@ -239,3 +239,54 @@ def test_errors():
         with pytest.raises(lbmp.LbmpError) as e:
             s.permeability_gradient(5)
         assert e.value.status == lbmp.ESTATE
+
+
+def _medium(nx, ny, seed):
+    r = np.random.RandomState(seed)
+    eps = 0.2 + 0.7 * r.rand(ny, nx)
+    eps[r.rand(ny, nx) < 0.05] = 0.0
+    return eps, 10.0 ** (3.0 * r.rand(ny, nx) - 1.0)
+
+
+def _grad(cfg, eps, k_i, nsteps, every):
+    with lbmp.Sim(cfg) as s:
+        s.set_fields(eps, k_i, np.zeros_like(eps))
+        _, gl, ge = s.permeability_gradient(nsteps, every, device=False)
+    return gl.numpy(), ge.numpy()
+
+
+@pytest.mark.parametrize("nx,ny,pressure", [(3, 5, 0), (33, 40, 0), (64, 17, 0), (131, 300, 0),
+                                            (3, 7, 1), (4, 33, 1), (66, 18, 1), (130, 300, 1)])
+def test_reverse_step_rolls_with_the_medium(nx, ny, pressure):
+    """A periodic box rolled in y (and x) gives the rolled gradient: the rows and
+    columns of a warp's part of the lattice fall differently, the arithmetic of a
+    node does not.  Between pressure columns only k_g's own FP64 sum is in another
+    order (its share in d/d eps, to 1e-12)."""
+    drive = dict(bc_x=lbmp.BCX_PRESSURE, rho_in=1.01, rho_out=0.99) if pressure else {}
+    cfg = lbmp.SimConfig(nx, ny, G=(1e-4, 2e-5), forchheimer=1, **drive)
+    eps, k_i = _medium(nx, ny, nx)
+    gl, ge = _grad(cfg, eps, k_i, 9, 4)
+    shift = (ny // 2 + 1, 0 if pressure else nx // 2)
+    roll = lambda f: np.ascontiguousarray(np.roll(f, shift, (0, 1)))
+    rl, re = _grad(cfg, roll(eps), roll(k_i), 9, 4)
+    assert np.abs(gl).max() > 0 and np.abs(ge).max() > 0
+    assert np.array_equal(rl, roll(gl))
+    if pressure:
+        assert np.abs(re - roll(ge)).max() <= 1e-12 * np.abs(ge).max()
+    else:
+        assert np.array_equal(re, roll(ge))
+
+
+@pytest.mark.parametrize("nx,ny,pressure,walls", [(1000, 520, 1, 1), (997, 530, 0, 1),
+                                                  (1300, 901, 1, 0), (64, 8200, 0, 0)])
+def test_recompute_two_steps_a_launch(nx, ny, pressure, walls):
+    """The levels recomputed two per launch are those of single steps: segments of
+    one step, and of odd and even lengths, give the same bits."""
+    drive = dict(bc_x=lbmp.BCX_PRESSURE, rho_in=1.01, rho_out=0.99) if pressure else {}
+    cfg = lbmp.SimConfig(nx, ny, G=(1e-4, 2e-5), forchheimer=walls,
+                         bc_y=lbmp.BCY_WALLS if walls else lbmp.BCY_PERIODIC, **drive)
+    eps, k_i = _medium(nx, ny, 3)
+    ref = _grad(cfg, eps, k_i, 7, 1)
+    for every in (2, 3, 7):
+        got = _grad(cfg, eps, k_i, 7, every)
+        assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
