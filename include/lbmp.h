@@ -63,8 +63,10 @@ typedef int32_t lbmp_status;
 #define LBMP_ROUND_NEAREST 1    /* round to nearest even */
 
 /* step kernel */
-#define LBMP_KERNEL_AUTO 0   /* the faster one measured on GB300: direct for FP32
-                                storage, staged for FP16 */
+#define LBMP_KERNEL_AUTO 0   /* the fastest one measured on GB300: several steps per
+                                launch on small lattices, two on large ones (and
+                                with FP16 storage), else direct for FP32 and
+                                staged for FP16; the same bits whichever runs */
 #define LBMP_KERNEL_STAGED 1 /* bulk copies into a shared-memory ring (persistent) */
 #define LBMP_KERNEL_DIRECT 2 /* one-pass loads from global memory */
 #define LBMP_KERNEL_WIDE 3   /* FP16 storage only: four consecutive nodes per thread,
@@ -103,8 +105,8 @@ typedef struct lbmp_params {
                            at the time level, its Kn = Kn(p0) p0 / p (the mean
                            free path of Eq. 10 is inversely proportional to p)
                            and k_a = k_i f_c(Kn) is formed at every step.
-                           FP32 storage needs the direct kernel, FP16 runs the
-                           staged one (AUTO) or the direct one; 1 + kn_beta
+                           FP32 storage runs under AUTO or the direct kernel,
+                           FP16 also under the staged one; 1 + kn_beta
                            (rho - rho0) must stay > 0 (checked for rho_in and
                            rho_out), else velocities turn non-finite (ENAN).
                            Not available to lbmp_batch_* and the adjoint. */
@@ -296,11 +298,12 @@ lbmp_status lbmp_permeability_gradient(lbmp_ctx *ctx, int64_t nsteps, int64_t ev
  * Batched sweeps.  `count` lattices of their own sizes (e.g. media
  * realizations x Knudsen numbers) share the physics parameters of p (tau, J,
  * G, boundary kinds, densities, Forchheimer, storage, rounding, seed; p->nx,
- * p->ny and p->kernel are ignored) and advance together: one launch per time
- * step covers a work list of row segments of all instances (one block per
- * segment, or a persistent grid walking it), or the tiles of all instances
- * in the staged bulk-copy kernel (CUDA graphs of 32 steps).  Each instance has its own populations, medium
- * and FP16 scale; the arithmetic per node is that of lbmp_step (Section III,
+ * p->ny and p->kernel are ignored) and advance together: one launch covers a
+ * work list of all instances for one time step (row segments, one block each
+ * or a persistent grid walking them, or the tiles of the staged bulk-copy
+ * kernel) or, beside that last shape, for two of them (strips of the two-step
+ * kernel); CUDA graphs of 32 launches.  Each instance has its own populations,
+ * medium and FP16 scale; the arithmetic per node is that of lbmp_step (Section III,
  * Eq. 12-17).  The launch shape (threads per block x nodes per thread x
  * grid mode) is chosen by lbmp_batch_tune.
  * --------------------------------------------------------------------- */

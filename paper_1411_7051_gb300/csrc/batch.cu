@@ -1,5 +1,5 @@
 // Batched sweeps: many lattices (media realizations, Knudsen numbers, sizes)
-// advanced together by one persistent launch per time step.
+// advanced together, one or two time steps per launch.
 //
 // Every instance has its own population buffers, medium and FP16 scale; the
 // physics parameters (tau, J, G, boundary kinds, densities, Forchheimer) are
@@ -8,7 +8,8 @@
 // BX * NPT nodes of instance item_inst[w].  Either one block per item, or a
 // persistent grid (SMs x resident blocks) walking contiguous item ranges.
 // The launch shape (BX, NPT, grid mode, or the staged bulk-copy kernel over
-// a tile list) is picked by lbmp_batch_tune, which times every candidate on
+// a tile list, beside which pairs of steps run the two-step kernel over a list of
+// strips) is picked by lbmp_batch_tune, which times every candidate on
 // the batch itself and restores the populations.
 // Per-instance global permeabilities are FP64 segmented reductions.
 #include <cuda_runtime.h>

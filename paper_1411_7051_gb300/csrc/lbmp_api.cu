@@ -361,9 +361,9 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
     }
     c->elem = (p.storage == LBMP_STORE_FP32) ? 4 : 2;
     c->sr = p.storage == LBMP_STORE_FP16 && p.fp16_rounding == LBMP_ROUND_STOCHASTIC;
-    // FP32: the direct kernel already saturates HBM (the staged one reaches
-    // ~0.95 of it); FP16 (static or dynamic Kn): the staged kernel issues
-    // fewer instructions per node.
+    // Single steps.  FP32: the direct kernel already saturates HBM (the staged
+    // one reaches ~0.95 of it); FP16 (static or dynamic Kn): the staged kernel
+    // issues fewer instructions per node.
     c->staged = p.kernel == LBMP_KERNEL_STAGED ||
                 (p.kernel == LBMP_KERNEL_AUTO && p.storage == LBMP_STORE_FP16);
     c->wide = p.kernel == LBMP_KERNEL_WIDE;
