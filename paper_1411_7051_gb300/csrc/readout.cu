@@ -293,7 +293,10 @@ __global__ void __launch_bounds__(kReadBX, kReadPerSM)
   __syncthreads();
   const PairIn<S> p(fin, med, a, blockIdx.x * kReadBX + threadIdx.x);
   const double umax = *umax_p;
-  const bool in_range = umax > 1e-20 && umax < 1e8;  // also false for infinity
+  // A non-finite velocity makes the maximum infinite and has no bin (its quotient is
+  // NaN, no index): nothing is counted, the caller reports the lattice.
+  if (!isfinite(umax)) return;
+  const bool in_range = umax > 1e-20 && umax < 1e8;
   const float per = in_range ? (float)nbins / ((float)umax * 0x1p30f) : 0.0f;
   int run_bin = 0;
   unsigned run = 0;
