@@ -335,15 +335,22 @@ __global__ void __launch_bounds__(batch_threads<S>(), 1)
   }
 }
 
+// The staged kernel's shared-memory limit, on the current device.
+template <class S, bool SR>
+static cudaError_t batch_staged_limit() {
+  return cudaFuncSetAttribute(batch_staged_kernel<S, SR>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, batch_smem_bytes<S>());
+}
+static cudaError_t prepare_batch_staged(int storage, bool sr) {
+  if (storage == LBMP_STORE_FP32) return batch_staged_limit<StoreF32, false>();
+  return sr ? batch_staged_limit<StoreF16, true>() : batch_staged_limit<StoreF16, false>();
+}
+
 template <class S, bool SR>
 static cudaError_t launch_batch_staged_t(const StepArgs &base, const BatchInst *inst,
                                          const int4 *tiles, int ntiles, int parity,
                                          const unsigned long long *tctr, int k, unsigned *err,
                                          int nsm, cudaStream_t s) {
-  static const cudaError_t attr = cudaFuncSetAttribute(
-      batch_staged_kernel<S, SR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-      batch_smem_bytes<S>());
-  if (attr != cudaSuccess) return attr;
   if (ntiles <= 0) return cudaSuccess;
   const int grid = ntiles < nsm ? ntiles : nsm;
   batch_staged_kernel<S, SR><<<grid, batch_threads<S>(), batch_smem_bytes<S>(), s>>>(
@@ -409,10 +416,7 @@ static cudaError_t launch_batch_fused_t(const StepArgs &base, const BatchInst *i
                                         const int4 *tasks, int ntasks, int parity,
                                         const unsigned long long *tctr, int k, cudaStream_t s) {
   using C = FusedCfg<S, Q, false>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(batch_fused_kernel<S, SR, FORCH, Q>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-  if (attr != cudaSuccess) return attr;
+  static_assert(C::kSmemBytes <= 48 * 1024, "within the limit that every kernel has");
   batch_fused_kernel<S, SR, FORCH, Q>
       <<<(ntasks + kFusedWarps - 1) / kFusedWarps, kFusedWarps * 32, C::kSmemBytes, s>>>(
           base, inst, tasks, ntasks, parity, tctr, k);
@@ -922,6 +926,11 @@ lbmp_status lbmp_batch_create(const lbmp_params *pin, int32_t count, const int32
     if (e != cudaSuccess) {
       delete b;
       return bcuda(e, "device query");
+    }
+    e = lbmp::prepare_batch_staged(p.storage, b->sr);
+    if (e != cudaSuccess) {
+      delete b;
+      return bcuda(e, "shared-memory limit of the staged kernel");
     }
     lbmp_status st = LBMP_OK;
 #define BTRY(x)           \

@@ -43,15 +43,27 @@ bool fused_covers(int storage, bool dyn, int nx, int ny) {
   return storage != 0 || (long long)nx * ny >= (dyn ? 1000000 : 500000);
 }
 
+// The kernel's shared-memory limit, on the current device, where it needs more than
+// the default 48 KB (FP32 with a dynamic Kn, two pairs a lane: 54 KB).
+constexpr int kDefaultSmem = 48 * 1024;
+cudaError_t prepare_fused(int storage, bool dyn, bool forch) {
+  using C = FusedCfg<StoreF32, 2, true>;
+  static_assert(FusedCfg<StoreF32, 2, false>::kSmemBytes <= kDefaultSmem &&
+                    FusedCfg<StoreF32, 1, true>::kSmemBytes <= kDefaultSmem &&
+                    FusedCfg<StoreF16, 2, true>::kSmemBytes <= kDefaultSmem,
+                "every other form fits the default limit");
+  if (storage != 0 || !dyn) return cudaSuccess;
+  return forch ? cudaFuncSetAttribute(fused_step_kernel<StoreF32, false, true, false, true, 2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes)
+               : cudaFuncSetAttribute(fused_step_kernel<StoreF32, false, true, false, false, 2>,
+                                      cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
+}
+
 template <class S, bool SR, bool DYN, bool MOM, bool FORCH, int Q>
 static cudaError_t launch_fused_q(const StepArgs &a, int rows, const void *fin, void *fout,
                                   const float2 *med, const unsigned long long *tctr, int k,
                                   const FusedPlan &plan, float *mom1, float *mom2, cudaStream_t s) {
   using C = FusedCfg<S, Q, DYN>;
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
-  if (attr != cudaSuccess) return attr;
   return launch_chained(fused_step_kernel<S, SR, DYN, MOM, FORCH, Q>,
                         dim3((plan.tasks + kFusedWarps - 1) / kFusedWarps), dim3(kFusedWarps * 32),
                         C::kSmemBytes, s,

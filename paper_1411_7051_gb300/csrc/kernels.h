@@ -73,7 +73,9 @@ cudaError_t launch_staged(int storage, bool sr, const StepArgs &a, int rows, con
 // single-step kernels (FP16 with stochastic rounding: of the staged one),
 // with the rounding bits of time levels *tctr + k and *tctr + k + 1.
 // fused_covers(): the lattices on which lbmp_step pairs its steps.
+// prepare_fused() raises the shared-memory limit of the kernel on the current device.
 bool fused_covers(int storage, bool dyn, int nx, int ny);
+cudaError_t prepare_fused(int storage, bool dyn, bool forch);
 cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                          void *fout, const float2 *med, const unsigned long long *tctr, int k,
                          int nsm, cudaStream_t s);
@@ -88,6 +90,7 @@ struct TilePlan {
 bool tile_covers(int storage, int nx, int rows);
 bool tile_plan(int storage, bool dyn, int nx, int rows, bool pressure, bool walls, int nsm,
                TilePlan *out);
+cudaError_t prepare_tile(int storage, bool sr, bool dyn, bool forch);  // as prepare_fused()
 cudaError_t launch_tile(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                         void *fout, const float2 *med, const unsigned long long *tctr, int k,
                         const TilePlan &p, int levels, cudaStream_t s);

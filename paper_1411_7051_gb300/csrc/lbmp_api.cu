@@ -389,6 +389,15 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
                  lbmp::tile_plan(p.storage, dyn, p.nx, c->rows(), p.bc_x == LBMP_BCX_PRESSURE,
                                  p.bc_y == LBMP_BCY_WALLS, c->nsm, &c->tile);
       if (c->tiled) c->fused = false;
+      // limits belong to a device: raised for every context, as the staged kernel's
+      if (c->tiled)
+        e = lbmp::prepare_tile(p.storage, c->sr, dyn, p.forchheimer != 0);
+      else if (c->fused)
+        e = lbmp::prepare_fused(p.storage, dyn, p.forchheimer != 0);
+      if (e != cudaSuccess) {
+        delete c;
+        return cuda_fail(e, "shared-memory limit of the step kernel");
+      }
     }
     lbmp_status st = LBMP_OK;
 #define LBMP_TRY(x)     \

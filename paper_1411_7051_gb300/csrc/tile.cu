@@ -56,15 +56,25 @@ bool tile_plan(int storage, bool dyn, int nx, int rows, bool pressure, bool wall
   return best > 0.0;
 }
 
+// The kernel's shared-memory limit, on the current device.
+template <class S, bool SR, bool DYN, bool FORCH>
+static cudaError_t tile_limit() {
+  return cudaFuncSetAttribute(tile_step_kernel<S, SR, DYN, FORCH>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              TileCfg<S, DYN>::kSmemBytes);
+}
+cudaError_t prepare_tile(int storage, bool sr, bool dyn, bool forch) {
+#define LBMP_TILE(S, SR, DYN) (forch ? tile_limit<S, SR, DYN, true>() : tile_limit<S, SR, DYN, false>())
+  if (storage == 0) return dyn ? LBMP_TILE(StoreF32, false, true) : LBMP_TILE(StoreF32, false, false);
+  if (sr) return dyn ? LBMP_TILE(StoreF16, true, true) : LBMP_TILE(StoreF16, true, false);
+  return dyn ? LBMP_TILE(StoreF16, false, true) : LBMP_TILE(StoreF16, false, false);
+#undef LBMP_TILE
+}
+
 template <class S, bool SR, bool DYN, bool FORCH>
 static cudaError_t launch_tile_t(const StepArgs &a, int rows, const void *fin, void *fout,
                                  const float2 *med, const unsigned long long *tctr, int k,
                                  const TilePlan &p, int levels, cudaStream_t s) {
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(tile_step_kernel<S, SR, DYN, FORCH>,
-                           cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           TileCfg<S, DYN>::kSmemBytes);
-  if (attr != cudaSuccess) return attr;
   const long long w = (a.nx + p.tx - 1) / p.tx + 2 * levels, h = (rows + p.ty - 1) / p.ty + 2 * levels;
   if (w * h > TileCfg<S, DYN>::kNodes || levels < 1 || levels > kTileMaxLevels)
     return cudaErrorInvalidValue;  // the block's shared memory holds kNodes nodes
