@@ -56,9 +56,10 @@ struct lbmp_ctx {
   int fault_alloc_at = 0;       // simulated allocation failure (testing)
   int drop_tile = -1;           // withheld tile of the staged kernel (testing)
   // step graphs: [l][cur] replays 2^l launches starting from buffer cur (of
-  // per_launch() steps each); odd[cur] the single step left over with `fused`
+  // per_launch() steps each); rest[n][cur] the n < per_launch() steps left over
+  static constexpr int kMaxPerLaunch = 16;
   cudaGraphExec_t graph[6][2] = {};
-  cudaGraphExec_t odd[2] = {};
+  cudaGraphExec_t rest[kMaxPerLaunch][2] = {};
 
   lbmp::StepArgs args() const {
     lbmp::StepArgs a;

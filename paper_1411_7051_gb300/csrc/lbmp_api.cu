@@ -92,11 +92,12 @@ void free_graphs(lbmp_ctx *c) {
         cudaGraphExecDestroy(g);
         g = nullptr;
       }
-  for (auto &g : c->odd)
-    if (g) {
-      cudaGraphExecDestroy(g);
-      g = nullptr;
-    }
+  for (auto &n : c->rest)
+    for (auto &g : n)
+      if (g) {
+        cudaGraphExecDestroy(g);
+        g = nullptr;
+      }
 }
 
 void release(lbmp_ctx *c) {
@@ -596,15 +597,10 @@ lbmp_status lbmp_step(lbmp_ctx *c, int64_t n) {
     }
     const int rest = (int)(n % per);
     if (rest > 0) {
-      if (c->tiled) {
-        LBMP_CK(launch_steps(c, c->args(), c->cur, rest, 0, c->stream));
-        if (c->sr) LBMP_CK(lbmp::launch_bump(c->d_tctr, rest, c->stream));
-      } else {
-        cudaGraphExec_t *slot = &c->odd[c->cur];
-        st = get_graph(c, slot, 1, 1, c->cur);
-        if (st) return st;
-        LBMP_CK(cudaGraphLaunch(*slot, c->stream));
-      }
+      cudaGraphExec_t *slot = &c->rest[rest][c->cur];
+      st = get_graph(c, slot, 1, rest, c->cur);
+      if (st) return st;
+      LBMP_CK(cudaGraphLaunch(*slot, c->stream));
       c->launches += 1 + (c->sr ? 1 : 0);
       c->cur ^= 1;
     }

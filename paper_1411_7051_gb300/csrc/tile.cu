@@ -3,10 +3,13 @@
 
 #include <algorithm>
 
+#include "context.h"
 #include "kernels.h"
 #include "tile.cuh"
 
 namespace lbmp {
+
+static_assert(kTileMaxLevels <= lbmp_ctx::kMaxPerLaunch, "a graph slot for every remainder");
 
 // Lattices that take it (us a step, before -> with it): FP32 up to some 170 000
 // nodes (64 x 33: 2.0 -> 1.2, 256^2 2.7 -> 1.9, 410 x 200 2.9 -> 2.1, 400^2 3.6 -> 2.9;
