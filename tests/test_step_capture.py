@@ -37,3 +37,17 @@ def test_capture_is_refused(L, nx, ny, kw, warm):
         assert (after.steps, after.launches) == (before.steps, before.launches)
         assert L.lbmp_step(h, n) == lbmp.OK
         L.lbmp_destroy(h)
+
+
+@pytest.mark.parametrize("nx,ny,direct", [(64, 33, 1), (40, 4000, 1), (128, 64, 2), (410, 200, 2),
+                                          (3000, 56, 2)])
+def test_few_steps_of_a_small_fp32_lattice_run_the_direct_kernel(L, nx, ny, direct):
+    """One step, and two on lattices that fill the direct kernel's blocks, cost
+    less without the halo of a tile."""
+    for n in (1, 2, 3):
+        st, h = fake.create(L, fake.params(nx, ny))
+        tile, step = (L.fake_launches(k) for k in (b"16tile_step_kernel", b"11step_kernel"))
+        assert L.lbmp_step(h, n) == lbmp.OK
+        assert L.fake_launches(b"16tile_step_kernel") == tile + (n > direct)
+        assert L.fake_launches(b"11step_kernel") == step + (n if n <= direct else 0)
+        L.lbmp_destroy(h)
