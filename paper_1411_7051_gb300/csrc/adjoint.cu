@@ -605,18 +605,17 @@ struct DevBuf {
 // The launches of one backward segment: n recompute steps from checkpoint ck
 // (the first step reads it in place, the two state buffers at segp then
 // alternate; level t's moments go to mom + t * mom_level; two steps per launch
-// on the lattices where that is the faster form), then the n reverse steps from
+// by the plan `pairs` unless that is null), then the n reverse steps from
 // the last level down, with an FP64 fold after every kFold-th reverse step of the
 // whole sweep (`reversed` of them done before this segment).  lam[0] holds
 // Lambda^{t+1} of the segment's last level on entry.  Adds its launches to
 // *launches.
 cudaError_t enqueue_segment(const lbmp::AdjArgs &A0, int rows, const float2 *med, const char *ck,
                             char *segp, size_t state, char *momp, size_t mom_level, int64_t n,
-                            float *const lam[2], int64_t reversed, int nsm, int64_t *launches,
-                            cudaStream_t s) {
+                            float *const lam[2], int64_t reversed, const lbmp::FusedPlan *pairs,
+                            int nsm, int64_t *launches, cudaStream_t s) {
   lbmp::AdjArgs A = A0;
   const lbmp::StepArgs &a = A.a;
-  const bool pairs = lbmp::fused_covers(LBMP_STORE_FP32, false, a.nx, a.ny);
   cudaError_t e = cudaSuccess;
   const float *in = (const float *)ck;
   int to = 0;
@@ -624,7 +623,7 @@ cudaError_t enqueue_segment(const lbmp::AdjArgs &A0, int rows, const float2 *med
     float *out = (float *)(segp + state * to);
     float *m0 = (float *)(momp + mom_level * t), *m1 = (float *)(momp + mom_level * (t + 1));
     if (pairs && t + 1 < n) {
-      e = lbmp::launch_fused_moments(a, rows, in, out, med, m0, m1, nsm, s);
+      e = lbmp::launch_fused_moments(a, rows, in, out, med, m0, m1, *pairs, s);
       t += 2;
     } else {
       e = lbmp::launch_step_moments(a, rows, in, out, med, m0, s);
@@ -746,11 +745,14 @@ extern "C" lbmp_status lbmp_permeability_gradient(lbmp_ctx *c, int64_t nsteps, i
     // (one per fold phase) was captured and instantiated to be replayed a few
     // times (64 x 64, 400 steps: 4.46 ms against 3.73).
     float *lams[2] = {lam0, lam1};  // lams[0]: Lambda^{t+1} of the next reverse step
+    const bool pairs = lbmp::fused_covers(LBMP_STORE_FP32, false, a.nx, a.ny);
+    lbmp::FusedPlan plan{};
+    if (pairs) plan = lbmp::fused_plan(LBMP_STORE_FP32, false, a.nx, rows, c->nsm);
     int64_t reversed = 0;          // the FP32 accumulators fold every kFold reverse steps
     for (int64_t sg = nseg - 1; sg >= 0; --sg) {
       const int64_t t0 = sg * every, n = std::min(every, nsteps - t0);
       ACK(enqueue_segment(A, rows, c->med, ckp + state * sg, segp, state, momp, mom_level, n, lams,
-                          reversed, c->nsm, &c->launches, s));
+                          reversed, pairs ? &plan : nullptr, c->nsm, &c->launches, s));
       reversed += n;
       if (n & 1) std::swap(lams[0], lams[1]);
     }

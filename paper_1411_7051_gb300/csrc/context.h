@@ -40,6 +40,7 @@ struct lbmp_ctx {
   bool staged = true;            // staged kernel (else direct or wide)
   bool wide = false;             // wide FP16 kernel
   bool fused = false;            // lbmp_step pairs its steps (two per launch)
+  lbmp::FusedPlan pairs{};
   bool tiled = false;            // ... or runs tile.levels of them per launch
   lbmp::TilePlan tile{};
   // steps of a full launch of lbmp_step

@@ -8,28 +8,43 @@
 
 namespace lbmp {
 
-struct FusedPlan {
-  FusedStrips f;
-  int seg, edges, tasks;  // rows per segment; edge warps, all warps
-};
+// The split of the smallest cost (fused_cost), of all splits into equal segments.
+// Many numbers of parts give one height: each height is looked at once (64 x 8192:
+// 180 of 8192 candidates, 71 -> 2 us).
 template <class C>
-static FusedPlan fused_plan(int nx, int rows, int nsm) {
+static FusedPlan split(int q, int nx, int rows, int nsm) {
   const double cap = (double)nsm * C::kBlocks * kFusedWarps;
-  FusedPlan best{fused_strips<C>(nx), rows, 0, 0};
-  const int most = (int)std::max(1.0, std::min((double)rows, 8.0 * cap / (best.f.inner + 1)));
+  const FusedStrips f = fused_strips<C>(nx);
+  FusedPlan best{q, rows, 0, 0};
+  const int most = (int)std::max(1.0, std::min((double)rows, 8.0 * cap / (f.inner + 1)));
   double best_cost = -1.0;
-  for (int parts = 1; parts <= most; ++parts) {
+  for (int parts = 1; parts <= most;) {
     const int seg = (rows + parts - 1) / parts;
     const int n = (rows + seg - 1) / seg;
-    const int edges = (n + best.f.per - 1) / best.f.per;
-    const int tasks = edges + best.f.inner * n;
+    const int edges = (n + f.per - 1) / f.per;
+    const int tasks = edges + f.inner * n;
     const double cost = fused_cost(seg, tasks / cap);
     if (best_cost < 0.0 || cost < best_cost) {
       best_cost = cost;
-      best = {best.f, seg, edges, tasks};
+      best = {q, seg, edges, tasks};
     }
+    if (seg == 1) break;
+    parts = (rows + seg - 2) / (seg - 1);  // the fewest of the next lower height
   }
   return best;
+}
+
+// Two pairs a lane spend fewer instructions a node, one pair a lane spreads a small
+// lattice over more warps: 768^2 FP32 7.8 / 7.2 us a step, 1024^2 10.2 / 10.5,
+// 1531 x 1153 14.1 / 17.0, 4096^2 108.5 / 119.
+FusedPlan fused_plan(int storage, bool dyn, int nx, int rows, int nsm) {
+  const bool wide = nx >= FusedCfg<StoreF32, 2, false>::kCols && (long long)nx * rows >= 1000000;
+#define LBMP_SPLIT(S, DYN)                                       \
+  (wide ? split<FusedCfg<S, 2, DYN>>(2, nx, rows, nsm)           \
+        : split<FusedCfg<S, 1, DYN>>(1, nx, rows, nsm))
+  if (storage == 0) return dyn ? LBMP_SPLIT(StoreF32, true) : LBMP_SPLIT(StoreF32, false);
+  return dyn ? LBMP_SPLIT(StoreF16, true) : LBMP_SPLIT(StoreF16, false);
+#undef LBMP_SPLIT
 }
 
 // Where two steps per launch are the faster form.  FP16 storage: everywhere
@@ -68,33 +83,26 @@ static cudaError_t launch_fused_q(const StepArgs &a, int rows, const void *fin, 
                         dim3((plan.tasks + kFusedWarps - 1) / kFusedWarps), dim3(kFusedWarps * 32),
                         C::kSmemBytes, s,
           a, (const typename S::T *)fin, (typename S::T *)fout, med, tctr, k, rows, plan.seg,
-          plan.f, plan.edges, plan.tasks, mom1, mom2);
+          fused_strips<C>(a.nx), plan.edges, plan.tasks, mom1, mom2);
 }
 
 template <class S, bool SR, bool DYN, bool MOM>
 static cudaError_t launch_fused_t(const StepArgs &a, int rows, const void *fin, void *fout,
                                   const float2 *med, const unsigned long long *tctr, int k,
-                                  int nsm, float *mom1, float *mom2, cudaStream_t s) {
-  using C1 = FusedCfg<S, 1, DYN>;
-  using C2 = FusedCfg<S, 2, DYN>;
-  // two pairs a lane spend fewer instructions a node, one pair a lane spreads
-  // a small lattice over more warps: 768^2 FP32 7.8 / 7.2 us a step, 1024^2
-  // 10.2 / 10.5, 1531 x 1153 14.1 / 17.0, 4096^2 108.5 / 119
-  const bool wide = a.nx >= C2::kCols && (long long)a.nx * rows >= 1000000;
-  const FusedPlan p = wide ? fused_plan<C2>(a.nx, rows, nsm) : fused_plan<C1>(a.nx, rows, nsm);
+                                  const FusedPlan &p, float *mom1, float *mom2, cudaStream_t s) {
 #define LBMP_FUSED(FORCH, Q) \
   launch_fused_q<S, SR, DYN, MOM, FORCH, Q>(a, rows, fin, fout, med, tctr, k, p, mom1, mom2, s)
-  if (a.forch) return wide ? LBMP_FUSED(true, 2) : LBMP_FUSED(true, 1);
-  return wide ? LBMP_FUSED(false, 2) : LBMP_FUSED(false, 1);
+  if (a.forch) return p.q == 2 ? LBMP_FUSED(true, 2) : LBMP_FUSED(true, 1);
+  return p.q == 2 ? LBMP_FUSED(false, 2) : LBMP_FUSED(false, 1);
 #undef LBMP_FUSED
 }
 
 cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                          void *fout, const float2 *med, const unsigned long long *tctr, int k,
-                         int nsm, cudaStream_t s) {
+                         const FusedPlan &plan, cudaStream_t s) {
   const bool dyn = a.kn0 != nullptr;
 #define LBMP_FUSED(S, SR, DYN) \
-  launch_fused_t<S, SR, DYN, false>(a, rows, fin, fout, med, tctr, k, nsm, nullptr, nullptr, s)
+  launch_fused_t<S, SR, DYN, false>(a, rows, fin, fout, med, tctr, k, plan, nullptr, nullptr, s)
   if (storage == 0)
     return dyn ? LBMP_FUSED(StoreF32, false, true) : LBMP_FUSED(StoreF32, false, false);
   if (sr) return dyn ? LBMP_FUSED(StoreF16, true, true) : LBMP_FUSED(StoreF16, true, false);
@@ -103,9 +111,9 @@ cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, cons
 }
 
 cudaError_t launch_fused_moments(const StepArgs &a, int rows, const float *fin, float *fout,
-                                 const float2 *med, float *mom1, float *mom2, int nsm,
-                                 cudaStream_t s) {
-  return launch_fused_t<StoreF32, false, false, true>(a, rows, fin, fout, med, nullptr, 0, nsm,
+                                 const float2 *med, float *mom1, float *mom2,
+                                 const FusedPlan &plan, cudaStream_t s) {
+  return launch_fused_t<StoreF32, false, false, true>(a, rows, fin, fout, med, nullptr, 0, plan,
                                                       mom1, mom2, s);
 }
 

@@ -52,11 +52,17 @@ cudaError_t launch_step(int storage, bool sr, const StepArgs &a, int rows, const
 // three [ny][pitch] float planes at mom, a.plane apart (adjoint recompute).
 cudaError_t launch_step_moments(const StepArgs &a, int rows, const float *fin, float *fout,
                                 const float2 *med, float *mom, cudaStream_t s);
+// The split of a two-step launch, made once per lattice (or gradient): node pairs
+// per lane, rows per segment, edge warps and all warps.
+struct FusedPlan {
+  int q, seg, edges, tasks;
+};
+FusedPlan fused_plan(int storage, bool dyn, int nx, int rows, int nsm);
 // Two such steps in one launch (fused.cuh): the moments of the two levels go
 // to mom1 and mom2.
 cudaError_t launch_fused_moments(const StepArgs &a, int rows, const float *fin, float *fout,
-                                 const float2 *med, float *mom1, float *mom2, int nsm,
-                                 cudaStream_t s);
+                                 const float2 *med, float *mom1, float *mom2,
+                                 const FusedPlan &plan, cudaStream_t s);
 // Vectorised FP16 variant of the same step (four nodes per thread).
 cudaError_t launch_wide(bool sr, const StepArgs &a, int rows, const void *fin, void *fout,
                         const float2 *med, const unsigned long long *tctr, int k,
@@ -78,7 +84,7 @@ bool fused_covers(int storage, bool dyn, int nx, int ny);
 cudaError_t prepare_fused(int storage, bool dyn, bool forch);
 cudaError_t launch_fused(int storage, bool sr, const StepArgs &a, int rows, const void *fin,
                          void *fout, const float2 *med, const unsigned long long *tctr, int k,
-                         int nsm, cudaStream_t s);
+                         const FusedPlan &plan, cudaStream_t s);
 // Several time steps in one launch of a small lattice (tile.cuh), bit for bit
 // those of the single-step kernels: `levels` <= plan.levels steps with the
 // rounding bits from time level *tctr + k on.  tile_covers(): the lattices that

@@ -182,7 +182,7 @@ cudaError_t launch_steps(lbmp_ctx *c, const StepArgs &a, int b, int n, int k, cu
                              c->d_tctr, k, c->tile, n, s);
   if (n == 2 && c->fused)
     return lbmp::launch_fused(c->p.storage, c->sr, a, c->rows(), c->buf[b], c->buf[b ^ 1], c->med,
-                              c->d_tctr, k, c->nsm, s);
+                              c->d_tctr, k, c->pairs, s);
   return launch_one(c, a, c->buf[b], c->buf[b ^ 1], k, s);
 }
 
@@ -390,6 +390,7 @@ lbmp_status lbmp_create(const lbmp_params *pin, lbmp_ctx **out) {
                  lbmp::tile_plan(p.storage, dyn, p.nx, c->rows(), p.bc_x == LBMP_BCX_PRESSURE,
                                  p.bc_y == LBMP_BCY_WALLS, c->nsm, &c->tile);
       if (c->tiled) c->fused = false;
+      if (c->fused) c->pairs = lbmp::fused_plan(p.storage, dyn, p.nx, c->rows(), c->nsm);
       // limits belong to a device: raised for every context, as the staged kernel's
       if (c->tiled)
         e = lbmp::prepare_tile(p.storage, c->sr, dyn, p.forchheimer != 0);
