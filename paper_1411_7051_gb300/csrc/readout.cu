@@ -24,11 +24,14 @@ constexpr int kReadPerSM = 4;  // resident blocks: 64 registers a thread
 // Columns in blocks of kReadBX, rows dealt out to the blocks of a column:
 // one wave of blocks, up to four (whose ends and starts overlap) while a thread
 // keeps at least 16 rows, which the block's own reduction needs to pay.  k_g, FP32:
-// 1024^2 37 us with one wave, 55 with four; 4096^2 210 and 186.
+// 1024^2 37 us with one wave, 55 with four; 4096^2 210 and 186.  Less than half a wave
+// beyond the first is left out, since the few blocks of it take as long as a whole
+// one: 40 x 65535 fields 282 us with 640 blocks, 172 with 608, populations 451 and
+// 263; 257 x 12000 137 with 753 blocks, 113 with 608.
 static dim3 read_grid(const StepArgs &a) {
   const long long wave = (long long)kReadPerSM * 152;
-  const long long blocks =
-      std::min(4 * wave, std::max(wave, (long long)a.nx * a.ny / (16 * kReadBX)));
+  long long blocks = std::min(4 * wave, (long long)a.nx * a.ny / (16 * kReadBX));
+  if (blocks < wave + wave / 2) blocks = wave;
   const int gx = (a.nx + kReadBX - 1) / kReadBX;
   return dim3(gx, (unsigned)std::max(1LL, std::min((long long)a.ny, blocks / gx)));
 }

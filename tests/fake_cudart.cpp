@@ -24,7 +24,7 @@ thread_local struct {
 int g_fail_attributes = 0;
 std::map<std::pair<int, const void *>, int> g_limit;
 std::map<const void *, std::string> g_name;
-std::map<std::string, long long> g_launches;
+std::map<std::string, long long> g_launches, g_blocks;
 std::map<void *, size_t> g_sizes;
 std::set<cudaStream_t> g_capturing;
 long long g_handles = 0;
@@ -34,11 +34,12 @@ cudaError_t done(cudaError_t e) {
   return e;
 }
 void *handle() { return (void *)(0x1000 + 16 * ++g_handles); }
-cudaError_t launch(const void *f, size_t smem) {
+cudaError_t launch(const void *f, dim3 grid, size_t smem) {
   auto it = g_limit.find({g_device, f});
   if (smem > (size_t)(it == g_limit.end() ? 48 * 1024 : it->second))
     return done(cudaErrorInvalidValue);
   ++g_launches[g_name[f]];
+  g_blocks[g_name[f]] = (long long)grid.x * grid.y * grid.z;
   return cudaSuccess;
 }
 cudaError_t copy(void *d, const void *s, size_t n, cudaMemcpyKind kind) {
@@ -63,6 +64,11 @@ long long fake_launches(const char *part) {
   for (const auto &l : g_launches)
     if (l.first.find(part) != std::string::npos) n += l.second;
   return n;
+}
+long long fake_blocks(const char *part) {  // of the last such launch
+  for (const auto &b : g_blocks)
+    if (b.first.find(part) != std::string::npos) return b.second;
+  return 0;
 }
 
 // ---- the runtime
@@ -145,7 +151,7 @@ cudaError_t cudaGetLastError(void) {
   return e;
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f, void **) {
-  return launch(f, c->dynamicSmemBytes);
+  return launch(f, c->gridDim, c->dynamicSmemBytes);
 }
 
 // ---- what nvcc's host code calls
@@ -164,8 +170,8 @@ cudaError_t __cudaGetKernel(cudaKernel_t *k, const void *f) {
   *k = (cudaKernel_t)f;
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t smem, cudaStream_t) {
-  return launch((const void *)k, smem);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 grid, dim3, void **, size_t smem, cudaStream_t) {
+  return launch((const void *)k, grid, smem);
 }
 void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
 void __cudaRegisterFatBinaryEnd(void **) {}

@@ -27,8 +27,9 @@ def load(directory):
         L = lbmp.load(out)
     finally:
         lbmp._lib = keep
-    L.fake_launches.restype = ctypes.c_longlong
-    L.fake_launches.argtypes = [ctypes.c_char_p]
+    for f in (L.fake_launches, L.fake_blocks):
+        f.restype = ctypes.c_longlong
+        f.argtypes = [ctypes.c_char_p]
     L.fake_capture.argtypes = [ctypes.c_void_p, ctypes.c_int]
     return L
 
