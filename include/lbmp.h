@@ -353,10 +353,12 @@ lbmp_status lbmp_batch_tune(lbmp_batch *b, int32_t steps, int32_t *chosen, doubl
  * timing, by every later batch of the same class (lbmp_batch_class): from
  * this process's cache, else from the file named by the environment
  * variable LBMP_TUNE_CACHE (lines "key shape ms_per_step", the last line of a
- * key wins).  On a miss it runs lbmp_batch_tune and stores the choice (and
- * appends it to that file).  *from_cache = 1 when nothing was timed; any of
- * the outputs may be NULL.  Cache file errors are ignored.  Errors: those of
- * lbmp_batch_tune on a miss. */
+ * key wins).  The key is the class, followed by "-p1" or "-p2" for a batch whose
+ * staged candidate advances two steps a launch (every instance at least 64
+ * columns wide and 6 rows high), by one or two node pairs a lane.  On a miss it
+ * runs lbmp_batch_tune and stores the choice (and appends it to that file).
+ * *from_cache = 1 when nothing was timed; any of the outputs may be NULL.  Cache
+ * file errors are ignored.  Errors: those of lbmp_batch_tune on a miss. */
 lbmp_status lbmp_batch_tune_cached(lbmp_batch *b, int32_t steps, int32_t *chosen,
                                    double *ms_per_step, int32_t *from_cache);
 /* Empty this process's shape cache (the file is left as it is). */

@@ -805,7 +805,8 @@ bool all_fields(const lbmp_batch *b) {
 // The launch shape tuned for one batch serves every later batch of the same
 // class: storage and rounding, boundary kinds, Forchheimer, the node-weighted
 // median of ceil(log2 nx) over the instances, floor(log2 of all nodes), and
-// the SM count of the device.  Kept per process, and in the file named by
+// the SM count of the device; the two-step launches, which some batches of a class
+// have beside the staged candidate, set them apart (tune_key).  Kept per process, and in the file named by
 // LBMP_TUNE_CACHE when that is set (one "key shape ms_per_step" line per
 // tuning; the last line of a key wins).  File errors are ignored: the cache
 // only saves tuning time.
@@ -837,6 +838,20 @@ std::string class_key(const lbmp_params &p, int count, const int32_t *nx, const 
   snprintf(buf, sizeof(buf), "s%d-r%d-x%d-y%d-f%d-n%d-t%d-m%d", (int)p.storage, sr, (int)p.bc_x,
            (int)p.bc_y, p.forchheimer ? 1 : 0, med, tcls, nsm);
   return buf;
+}
+
+// The key of a batch's entry: its class, and the node pairs per lane of its two-step
+// launches.  A shape timed without them says nothing about a batch that has them:
+// FP32 sweeps then kept a direct shape at 139 us a step instead of 84.
+std::string tune_key(const lbmp_batch *b) {
+  std::vector<int32_t> nx(b->count), ny(b->count);
+  for (int i = 0; i < b->count; ++i) {
+    nx[i] = b->h_inst[i].a.nx;
+    ny[i] = b->h_inst[i].a.ny;
+  }
+  std::string key = class_key(b->p, b->count, nx.data(), ny.data(), b->nsm);
+  if (b->ntasks > 0) key += b->fused_q == 2 ? "-p2" : "-p1";
+  return key;
 }
 
 struct TuneEntry {
@@ -1237,12 +1252,7 @@ lbmp_status lbmp_batch_tune_cached(lbmp_batch *b, int32_t steps, int32_t *chosen
   try {
     if (!b) return bfail(LBMP_EINVAL, "NULL batch");
     if (steps < 1) return bfail(LBMP_EINVAL, "steps must be >= 1");
-    std::vector<int32_t> nx(b->count), ny(b->count);
-    for (int i = 0; i < b->count; ++i) {
-      nx[i] = b->h_inst[i].a.nx;
-      ny[i] = b->h_inst[i].a.ny;
-    }
-    const std::string key = class_key(b->p, b->count, nx.data(), ny.data(), b->nsm);
+    const std::string key = tune_key(b);
     TuneEntry e{};
     bool hit;
     {

@@ -25,6 +25,8 @@ int g_fail_attributes = 0;
 std::map<std::pair<int, const void *>, int> g_limit;
 std::map<const void *, std::string> g_name;
 std::map<std::string, long long> g_launches, g_blocks;
+long long g_total = 0;
+std::map<cudaEvent_t, long long> g_events;
 std::map<void *, size_t> g_sizes;
 std::set<cudaStream_t> g_capturing;
 long long g_handles = 0;
@@ -38,6 +40,7 @@ cudaError_t launch(const void *f, dim3 grid, size_t smem) {
   auto it = g_limit.find({g_device, f});
   if (smem > (size_t)(it == g_limit.end() ? 48 * 1024 : it->second))
     return done(cudaErrorInvalidValue);
+  ++g_total;
   ++g_launches[g_name[f]];
   g_blocks[g_name[f]] = (long long)grid.x * grid.y * grid.z;
   return cudaSuccess;
@@ -138,10 +141,10 @@ cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) {
 }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = (cudaEvent_t)handle(); return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { g_events[e] = g_total; return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) {
-  *ms = 1.0f;
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b) {
+  *ms = (float)(g_events[b] - g_events[a]);  // a launch takes a millisecond
   return cudaSuccess;
 }
 const char *cudaGetErrorString(cudaError_t e) { return e == cudaSuccess ? "no error" : "fake error"; }
