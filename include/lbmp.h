@@ -345,9 +345,10 @@ lbmp_status lbmp_batch_synchronize(lbmp_batch *b);
 lbmp_status lbmp_batch_permeability(lbmp_batch *b, double *k_g, double *u_mean);
 /* Post-stream populations of instance i, [9][ny_i][nx_i] float64. */
 lbmp_status lbmp_batch_populations(lbmp_batch *b, int32_t i, double *f, int32_t where);
-/* Autotuner: time `steps` steps of every candidate launch shape on this
- * batch, keep the fastest, restore the populations and time level.  Returns
- * the chosen candidate index and its time per step (either may be NULL). */
+/* Autotuner: time `steps` steps (the next even number where the staged candidate
+ * advances two a launch) of every candidate launch shape on this batch, keep the
+ * fastest, restore the populations and time level.  Returns the chosen candidate
+ * index and its time per step (either may be NULL). */
 lbmp_status lbmp_batch_tune(lbmp_batch *b, int32_t steps, int32_t *chosen, double *ms_per_step);
 /* Autotuner with a cache.  The shape tuned for a batch is reused, without
  * timing, by every later batch of the same class (lbmp_batch_class): from

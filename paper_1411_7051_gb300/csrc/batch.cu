@@ -1385,6 +1385,8 @@ lbmp_status lbmp_batch_tune(lbmp_batch *b, int32_t steps, int32_t *chosen, doubl
     if (!all_fields(b)) return bfail(LBMP_ESTATE, "every instance needs its fields");
     const DeviceScope device_scope(b->device);
     BCK(device_scope.err);
+    // whole pairs: one step alone would time a kernel that a run hardly uses
+    if (b->ntasks > 0 && steps < INT32_MAX) steps += steps & 1;
     const size_t elem = b->p.storage == LBMP_STORE_FP32 ? 4 : 2;
     // save the current populations and the counter of every instance
     std::vector<void *> saved(b->count, nullptr);

@@ -1,6 +1,7 @@
 """The batch autotuner and the two-step launches beside its staged candidate: a
-shape tuned with them serves no batch without them, nor the reverse.  Host logic,
-against a runtime without a GPU (a launch takes a millisecond there)."""
+shape tuned with them serves no batch without them, nor the reverse, and the
+tuner times them whatever the number of steps.  Host logic, against a runtime
+without a GPU (a launch takes a millisecond there)."""
 import ctypes
 
 import pytest
@@ -51,3 +52,8 @@ def test_batches_with_and_without_pairs_are_tuned_apart(L, tmp_path, monkeypatch
     path.write_text(f"{key} 3 0.5\n")
     assert _tune(L, narrow) == (3, 1)
     assert _tune(L, pairs) == (STAGED, 0)
+
+
+@pytest.mark.parametrize("steps", [1, 2, 3])
+def test_the_tuner_times_pairs(L, steps):
+    assert _tune(L, PAIRS2, steps) == (STAGED, 0)
