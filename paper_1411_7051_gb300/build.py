@@ -44,9 +44,15 @@ def source_hash() -> str:
     return h.hexdigest()[:16]
 
 
-STEP_KERNEL_FILES = ["kernels.cu", "chain.cuh", "fused.cu", "fused.cuh", "kernels.h", "lattice.cuh", "staged.cuh"]
-ADJOINT_KERNEL_FILES = ["adjoint.cu", "kernels.h", "lattice.cuh"]
-BATCH_KERNEL_FILES = ["batch.cu", "fused.cuh", "kernels.h", "lattice.cuh", "staged.cuh"]
+# The sources of the kernels whose committed figures carry a hash: their translation
+# units (the adjoint's recompute runs the step kernels) and all that these include.
+STEP_KERNEL_FILES = ["kernels.cu", "fused.cu", "tile.cu", "chain.cuh", "fused.cuh", "kernels.h",
+                     "lattice.cuh", "pairs.cuh", "staged.cuh", "tile.cuh", "wide.cuh"]
+ADJOINT_KERNEL_FILES = ["adjoint.cu", "kernels.cu", "fused.cu", "chain.cuh", "fused.cuh", "kernels.h",
+                        "lattice.cuh", "pairs.cuh", "staged.cuh", "wide.cuh"]
+BATCH_KERNEL_FILES = ["batch.cu", "chain.cuh", "fused.cuh", "kernels.h", "lattice.cuh",
+                      "readout.cuh", "staged.cuh"]
+
 
 
 def kernel_hash(files=STEP_KERNEL_FILES) -> str:
