@@ -748,8 +748,8 @@ def batch_measure(lbmp, torch, n_media: int, n_kn: int, storage: str, K: int, W:
 
 def batch_roofline(r, K, peak, kind, storage):
     """Roofline of the batched step; `traffic` from the committed ncu figures
-    when they were taken on the current batched-kernel sources and on the
-    same set of instances (the same node count)."""
+    when they were taken on the current batched-kernel sources, on the same
+    set of instances (the same node count) and on launches of as many steps."""
     from paper_1411_7051_gb300 import build as lbuild
     spl = steps_per_launch(r.get("launches", K), K)
     per_launch_s = r["ms"] * 1e-3 / K * spl
@@ -758,6 +758,8 @@ def batch_roofline(r, K, peak, kind, storage):
     if r["staged"]:
         tr = profiled_traffic(f"batch_{storage}", lbuild.kernel_hash(lbuild.BATCH_KERNEL_FILES))
         if tr and tr.get("nodes") != r["nodes"]:
+            tr = None
+        if tr and "launches" in r and tr.get("steps_per_launch", 1) != spl:
             tr = None
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_kind": f"of {kind}",
