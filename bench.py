@@ -390,12 +390,17 @@ def whole_job_glups(world_size: int, nodes_per_rank: int, steps: int, ms_slowest
 
 
 def steps_per_launch(launches: int, steps: int) -> int:
-    """Time steps a kernel launch advanced: 2 when the run paired its steps
-    (launches: of the timed region, the few counter bumps included)."""
-    return 2 if launches < 0.75 * steps else 1
+    """Time steps a kernel launch advanced (launches: of the timed region, the
+    few counter bumps included): 1, 2 when the run paired its steps, or the mean
+    on a small lattice, whose launches take 4 to 16."""
+    if launches >= 0.75 * steps:
+        return 1
+    return 2 if launches >= 0.375 * steps else round(steps / launches)
 
 
 def kernel_name(kernel: str, tag: str, spl: int = 1) -> str:
+    if spl > 2:
+        return f"lbmp::tile_step_kernel<{tag}>"
     if spl == 2:
         return f"lbmp::fused_step_kernel<{tag}>"
     staged = kernel == "staged" or (kernel == "auto" and tag == "StoreF16")
@@ -450,7 +455,7 @@ def run_ours(args, ws, rank, local):
 
     def roofline(r, tag):
         spl = steps_per_launch(r["launches"], K)
-        per_launch_s = r["ms"] * 1e-3 / K * spl    # one launch per time step or two
+        per_launch_s = r["ms"] * 1e-3 / K * spl    # a launch takes spl time steps
         alg = r["bpu"] * r["nodes"]                 # bytes a launch reads and writes once
         achieved = alg / per_launch_s / 1e9
         tr = profiled_traffic(tag, src)
