@@ -302,7 +302,7 @@ lbmp_status lbmp_permeability_gradient(lbmp_ctx *ctx, int64_t nsteps, int64_t ev
  * work list of all instances for one time step (row segments, one block each
  * or a persistent grid walking them, or the tiles of the staged bulk-copy
  * kernel) or, beside that last shape, for two of them (strips of the two-step
- * kernel); CUDA graphs of 32 launches.  Each instance has its own populations,
+ * kernel); CUDA graphs of 32 steps.  Each instance has its own populations,
  * medium and FP16 scale; the arithmetic per node is that of lbmp_step (Section III,
  * Eq. 12-17).  The launch shape (threads per block x nodes per thread x
  * grid mode) is chosen by lbmp_batch_tune.

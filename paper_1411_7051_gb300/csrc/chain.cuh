@@ -7,8 +7,12 @@
 //
 // Every kernel launched this way calls chain_wait() before its first access to
 // memory that an earlier kernel of the stream writes (or reads: it may be
-// written here), so nothing is read early.  Such memory is not read through the
-// non-coherent path: those loads could be moved above the wait.
+// written here), so nothing is read early.  Populations, moments and adjoints, which
+// the kernels of a chain write, are not read through the non-coherent path: those
+// loads could be moved above the wait.  The medium is (__ldg, const __restrict__):
+// the calls that write it (lbmp_set_fields, lbmp_batch_set_fields) wait for the stream
+// before they return, so no kernel of a chain runs beside its writer.  A path that
+// queued a step behind the medium's kernels would have to give that up.
 #pragma once
 
 #include <cuda_runtime.h>

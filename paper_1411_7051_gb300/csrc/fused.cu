@@ -10,7 +10,7 @@ namespace lbmp {
 
 // The split of the smallest cost (fused_cost), of all splits into equal segments.
 // Many numbers of parts give one height: each height is looked at once (64 x 8192:
-// 180 of 8192 candidates, 71 -> 2 us).
+// 181 of 8192 candidates, 71 -> 2.3 us).
 template <class C>
 static FusedPlan split(int q, int nx, int rows, int nsm) {
   const double cap = (double)nsm * C::kBlocks * kFusedWarps;
@@ -35,8 +35,8 @@ static FusedPlan split(int q, int nx, int rows, int nsm) {
 }
 
 // Two pairs a lane spend fewer instructions a node, one pair a lane spreads a small
-// lattice over more warps: 768^2 FP32 7.8 / 7.2 us a step, 1024^2 10.2 / 10.5,
-// 1531 x 1153 14.1 / 17.0, 4096^2 108.5 / 119.
+// lattice over more warps: 768^2 FP32 7.2 / 7.0 us a step, 1024^2 9.8 / 10.1,
+// 1531 x 1153 13.9 / 14.6, 4096^2 113.8 / 114.8, FP16 96.7 / 112.9.
 FusedPlan fused_plan(int storage, bool dyn, int nx, int rows, int nsm) {
   const bool wide = nx >= FusedCfg<StoreF32, 2, false>::kCols && (long long)nx * rows >= 1000000;
 #define LBMP_SPLIT(S, DYN)                                       \
@@ -48,11 +48,10 @@ FusedPlan fused_plan(int storage, bool dyn, int nx, int rows, int nsm) {
 }
 
 // Where two steps per launch are the faster form.  FP16 storage: everywhere
-// (against the staged kernel 64 x 33: 9.8 -> 2.4 us a step, 512^2 6.4 -> 4.7,
-// 4096^2 112.5 -> 97).  FP32: the direct kernel needs fewer rows in a row on
-// small lattices (512^2: 4.5 us against 4.7; 768^2: 7.6 against 7.2; 4096^2: 190
-// against 113), with a dynamic Kn up to about 10^6 nodes (768^2: 8.8 against 10.0;
-// 1024^2: 13.5 against 11.8).
+// (against the staged kernel 512^2 6.4 -> 4.2 us a step, 4096^2 112 -> 97).  FP32:
+// the direct kernel needs fewer rows in a row on small lattices (512^2: 3.9 us
+// against 4.0; 768^2: 7.1 against 7.0; 4096^2: 190 against 114), with a dynamic Kn
+// up to about 10^6 nodes (768^2: 8.3 against 8.9; 1024^2: 13.3 against 11.4).
 bool fused_covers(int storage, bool dyn, int nx, int ny) {
   if (nx < FusedCfg<StoreF32, 1, false>::kCols || ny < kFusedMinNy) return false;
   return storage != 0 || (long long)nx * ny >= (dyn ? 1000000 : 500000);

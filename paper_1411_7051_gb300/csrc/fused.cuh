@@ -20,8 +20,9 @@
 // lane where nx is even, one node (half the segments) where it is odd.
 //
 // Bound: FP32 by HBM (40 B an update, 4096^2: 190 us a step with one step per
-// pass, 110 - 114 now, 0.87 of the copy bandwidth), FP16 by the issue of some
-// 265 instructions a pair and step (112.5 -> 97 us).
+// pass, 114 now, 0.87 of the copy bandwidth), FP16 by the issue of some
+// 300 instructions a pair and step and too few warps to cover their latency
+// (12 an SM; 112 -> 97 us).
 //
 // Every node is updated with the operations of the single-step kernels, in
 // their order and with their stochastic-rounding bits, so the populations
@@ -53,7 +54,7 @@ struct FusedCfg {
   static constexpr int kCols = 64 * Q;
   // Columns a strip stores: all but two at each side, or for FP32 with two
   // pairs per lane those of lanes 1 .. 30, whose rows start on 32-byte sectors
-  // (4096^2: 110 - 114 us a step against 118 with 124 columns).
+  // (4096^2: 114 us a step against 120 with 124 columns).
   static constexpr int kOut = sizeof(T) == 4 && Q == 2 ? 120 : kCols - 4;
   static constexpr int kLead = (kCols - kOut) / 2;
   static constexpr int kAlign = sizeof(T) == 4 && Q == 2 ? 8 : 4;  // of first columns
@@ -569,7 +570,7 @@ __device__ __forceinline__ void level_row(typename LaneRaw<S, float2>::R t[9][Q]
 }
 
 // The walk of an interior strip (first column c0) over rows [s0, s1), as
-// fused_walk, with the rows of level t copied ahead.
+// fused_edges, with the rows of level t copied ahead.
 template <class S, bool SR, bool DYN, bool MOM, int Q>
 __device__ __forceinline__ void fused_strip(const StepArgs &a, const typename S::T *fin,
                                             typename S::T *__restrict__ fout,
@@ -766,8 +767,8 @@ __host__ __device__ inline FusedStrips fused_strips(int nx) {
 // redundant rows and large ones leave the last wave uneven: up to one wave
 // 0.7 + w / 2 (a partly filled chip runs each row faster), 2.2 up to two, w + 0.25
 // beyond and a little more where the last wave is nearly empty.  Fitted to
-// sweeps of seg at 512^2 .. 4096^2 (1024^2: 6 rows 10.2 us a step, 5 rows 11.8;
-// 4096^2 FP32: 20 and 28 rows 110.5, 25 rows 113, one wave of 82 rows 121).
+// sweeps of seg at 512^2 .. 4096^2 (1024^2: 6 rows 9.8 us a step, 5 rows 11.4;
+// 4096^2 FP32: 20 and 28 rows 111, 26 rows 114, one wave of 82 rows 121).
 inline double fused_cost(int seg, double w) {
   if (w <= 1.0) return (seg + 2) * (0.7 + 0.5 * w);
   if (w <= 2.0) return (seg + 2) * 2.2;

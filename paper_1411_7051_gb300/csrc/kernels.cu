@@ -118,7 +118,6 @@ cudaError_t launch_step(int storage, bool sr, const StepArgs &a, int rows, const
     else
       return launch_chained(step_kernel<StoreF16, false, false>, grid, block, 0, s, a, f16i, f16o, med, tctr, k, nullptr);
   }
-  return cudaGetLastError();
 }
 
 cudaError_t launch_step_moments(const StepArgs &a, int rows, const float *fin, float *fout,

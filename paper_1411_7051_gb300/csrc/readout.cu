@@ -26,8 +26,8 @@ constexpr int kReadPerSM = 4;  // resident blocks: 64 registers a thread
 // keeps at least 16 rows, which the block's own reduction needs to pay.  k_g, FP32:
 // 1024^2 37 us with one wave, 55 with four; 4096^2 210 and 186.  Less than half a wave
 // beyond the first is left out, since the few blocks of it take as long as a whole
-// one: 40 x 65535 fields 282 us with 640 blocks, 172 with 608, populations 451 and
-// 263; 257 x 12000 137 with 753 blocks, 113 with 608.
+// one: 40 x 65535 fields 282 us with 640 blocks, 168 with 608, populations 447 and
+// 262; 257 x 12000 fields 134 with 753 blocks, 108 with 608.
 static dim3 read_grid(const StepArgs &a) {
   const long long wave = (long long)kReadPerSM * 152;
   long long blocks = std::min(4 * wave, (long long)a.nx * a.ny / (16 * kReadBX));
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(kReadBX, kReadPerSM)
 // 1 / (double)v, correctly rounded, for a positive normal v, by long division
 // in 32-bit integers: with v = m 2^(E - 150), m of 24 bits, the 53-bit quotient
 // 2^76 / m is formed 26 bits at a time from an FP32 reciprocal and exact
-// remainders.  (An FP64 division per node took 196 us at 4096^2.)
+// remainders.  (An FP64 division per node took 196 us at 4096^2, this 88.)
 static __device__ __noinline__ double wide_reciprocal_any(float v) { return 1.0 / (double)v; }
 __device__ __forceinline__ double wide_reciprocal(float v) {
   const uint32_t u = __float_as_uint(v), E = u >> 23;
